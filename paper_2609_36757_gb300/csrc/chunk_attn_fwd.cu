@@ -569,31 +569,17 @@ __device__ __forceinline__ float acc_total(const uint64_t (&acc)[4]) {
   return ((a0 + a1) + (b0 + b1)) + ((c0 + c1) + (d0 + d1));
 }
 
-// Mask columns >= valid of s[c] (the ragged end of a segment) and fold the
-// row max of s[c] into four independent accumulators.
-__device__ __forceinline__ void mask_max32(uint32_t (&sc)[32], int c, int valid,
-                                           float (&mx)[4]) {
-  if (valid < (c + 1) * 32) {
+// Mask the columns of s[c] outside [lo, hi) (relative to the tile).
+__device__ __forceinline__ void mask32(uint32_t (&sc)[32], int c, int lo,
+                                       int hi) {
 #pragma unroll
-    for (int i = 0; i < 32; ++i)
-      if (c * 32 + i >= valid) sc[i] = 0xff800000u;  // -inf
-  }
-#pragma unroll
-  for (int i = 0; i < 16; ++i)
-    mx[i & 3] = max3(mx[i & 3], __uint_as_float(sc[2 * i]),
-                     __uint_as_float(sc[2 * i + 1]));
+  for (int i = 0; i < 32; ++i)
+    if (c * 32 + i < lo || c * 32 + i >= hi) sc[i] = 0xff800000u;  // -inf
 }
 
-// One-shot: mask the columns of s[c] outside this row's visible range
-// [lo, hi) (relative to the tile) and fold the row max as mask_max32 does.
-__device__ __forceinline__ void mask_range_max32(uint32_t (&sc)[32], int c,
-                                                 int lo, int hi,
-                                                 float (&mx)[4]) {
-  if (lo > c * 32 || hi < (c + 1) * 32) {
-#pragma unroll
-    for (int i = 0; i < 32; ++i)
-      if (c * 32 + i < lo || c * 32 + i >= hi) sc[i] = 0xff800000u;  // -inf
-  }
+// Fold the row max of s[c] into four independent accumulators.
+__device__ __forceinline__ void max32(const uint32_t (&sc)[32],
+                                      float (&mx)[4]) {
 #pragma unroll
   for (int i = 0; i < 16; ++i)
     mx[i & 3] = max3(mx[i & 3], __uint_as_float(sc[2 * i]),
@@ -631,13 +617,28 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
     vis_lo = p.window < 0 ? 0 : max(0, c - p.window) * p.chunk_tokens;
     vis_hi = min((c + 1) * p.chunk_tokens, p.seq_tokens);
   }
+  // Few tiles need a mask: streaming, the ragged ends of the two segments (at
+  // most one tile each); one-shot, tiles that cross a chunk edge.  Whether
+  // this one does is settled before S is waited for and decided once per
+  // tile: worked out after the wait, with a test per 32 columns, it stood in
+  // the chain from S to P (480p ring, 84 CTAs of 63 tiles: 76.7 -> 75.6 us).
+  const int rag0_n = p.seg_len[0] % kBN, rag1_n = p.seg_len[1] % kBN;
+  const int rag0 = rag0_n ? p.seg_tiles0 - 1 - j0 : -1;
+  const int rag1 = rag1_n ? p.total_tiles - 1 - j0 : -1;
   for (int j = 0; j < n; ++j) {
-    int seg, tok0, valid;
     const int jt = rev ? n - 1 - j : j;  // the producers' order
-    if (kOneShot)
-      oneshot_tile(kv0, kv1, jt, seg, tok0, valid);
-    else
-      tile_coord(p, j0 + jt, seg, tok0, valid);
+    int lo = 0, hi = kBN;  // the columns of the tile that the row sees
+    bool masked;
+    if (kOneShot) {
+      const int tok0 = kv0 + jt * kBN;
+      lo = vis_lo - tok0;
+      hi = min(vis_hi, kv1) - tok0;
+      masked = __any_sync(0xffffffffu, lo > 0 || hi < kBN);
+    } else {
+      masked = jt == rag0 || jt == rag1;
+      if (jt == rag0) hi = rag0_n;
+      if (jt == rag1) hi = rag1_n;
+    }
     if (!(ok = wait_bar(&S->s_full[t], j & 1, S, p.status))) break;
     tc_fence_after();
     uint32_t s[4][32];
@@ -651,15 +652,12 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
       ++s_arrived;
     }
     float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
-    if (kOneShot) {
-      const int lo = vis_lo - tok0;
-      const int hi = min(vis_hi - tok0, valid);
+    if (masked) {
 #pragma unroll
-      for (int c = 0; c < 4; ++c) mask_range_max32(s[c], c, lo, hi, mx);
-    } else {
-#pragma unroll
-      for (int c = 0; c < 4; ++c) mask_max32(s[c], c, valid, mx);
+      for (int c = 0; c < 4; ++c) mask32(s[c], c, lo, hi);
     }
+#pragma unroll
+    for (int c = 0; c < 4; ++c) max32(s[c], mx);
     const float mrow = fmaxf(max3(mx[0], mx[1], mx[2]), mx[3]) * sl2;
     // The reference moves only when a row max passes it by more than the
     // threshold (decided per warp: TMEM accesses are warp-wide).
