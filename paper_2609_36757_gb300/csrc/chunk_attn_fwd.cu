@@ -21,7 +21,8 @@
 //   warps 0-3   softmax of query tile 0, one thread per row (TMEM lane);
 //   warps 4-7   softmax of query tile 1.
 // TMEM (512 columns): S (shared by the two tiles) | P_0 | P_1 | O_0 | O_1,
-// 128 + 64 + 64 + 128 + 128 columns.  S only lives until the softmax warps
+// 128 + 64 + 64 + 128 + 128 columns (d = 64: S_0 | S_1 | P_0 | P_1 | O_0 |
+// O_1, 128 + 128 + 4 x 64).  S only lives until the softmax warps
 // have loaded it (they release it before the row max), so the next QK^T of
 // either tile can follow at once; each tile's PV runs one key tile behind,
 // which gives its softmax three MMA steps to store P_t.  The MMA warp never
@@ -69,11 +70,29 @@ constexpr int kThreads = 384;   // 8 softmax warps, K and V producers, MMA,
                                 // relay
 constexpr int kBox = 128 * 128; // one TMA box: 128 rows x 64 bf16 (bytes)
 constexpr uint32_t kTmemCols = 512;
-// TMEM columns: one S tile shared by the two query tiles, P_0 and P_1 (bf16
-// pairs, 64 columns each), O_0 and O_1.
-constexpr uint32_t kTmemS = 0;
-constexpr uint32_t kTmemP = 128;
-constexpr uint32_t kTmemO = 256;
+// TMEM columns.  d = 128: one S tile shared by the two query tiles, P_0 and
+// P_1 (bf16 pairs, 64 columns each), O_0 and O_1 (128 columns each), all 512.
+// d = 64: O needs half the columns, and each query tile has an S of its own:
+// its QK^T then waits for its own softmax alone, which keeps the two tiles'
+// softmax warps apart in time (with a shared S each tile's S came a whole
+// hand-off after the other tile had read its own; d = 64 chunk step, 48 heads
+// of 3465 x 10395: 429.2 -> 415.4 us together with the early look at p_free).
+template <int D>
+struct Tmem {
+  static constexpr bool kOwnS = D == 64;
+  __host__ __device__ static constexpr uint32_t s(int t) {
+    return kOwnS ? t * 128u : 0u;
+  }
+  __host__ __device__ static constexpr uint32_t p(int t) {
+    return (kOwnS ? 256u : 128u) + t * 64u;
+  }
+  __host__ __device__ static constexpr uint32_t o(int t) {
+    return kOwnS ? 384u + t * 64u : 256u + t * 128u;
+  }
+};
+static_assert(Tmem<128>::o(1) + 128 == kTmemCols &&
+                  Tmem<64>::o(1) + 64 == kTmemCols,
+              "TMEM columns");
 constexpr float kRescaleThreshold = 8.0f;      // log2 units
 constexpr int kMinTilesPerPart = 4;             // key tiles per split part
 constexpr uint64_t kDefaultWaitLimitNs = 4000000000ull;  // 4 s per wait
@@ -91,6 +110,8 @@ constexpr int kRelay = 2 * 32;
 // Named barrier of a query tile's four softmax warps: their rows of O are
 // staged for the tile's TMA store.
 constexpr int kBarOStaged0 = 9;  // + t
+// "S read" of query tile 1 where each tile has an S of its own (d = 64).
+constexpr int kBarSFree1 = 11;
 
 struct TcParams {
   CUtensorMap q_map;                  // {d, Lq, H, B}
@@ -417,6 +438,7 @@ template <int D>
 __device__ void mma_issuer(const TcParams& p, uint8_t* smem, Shared* S,
                            uint32_t tmem, const Work& w) {
   using L = Layout<D>;
+  using T = Tmem<D>;
   constexpr uint32_t kIdescQK = idesc_bf16_f32(kBM, kBN, 0);
   constexpr uint32_t kIdescPV = idesc_bf16_f32(kBM, D, 1);
   const uint32_t sbase = smem_addr(smem);
@@ -433,7 +455,7 @@ __device__ void mma_issuer(const TcParams& p, uint8_t* smem, Shared* S,
   const uint32_t k_lo = desc_lo(sbase + L::k(0, 0), 16);
   const uint32_t v_lo = desc_lo(sbase + L::v(0, 0), kBox);
   constexpr uint32_t kStage16 = (uint32_t)(L::kNB * kBox) >> 4;
-  // S = Q_t K^T into the shared S columns: both operands K-major, 128-byte
+  // S_t = Q_t K^T: both operands K-major, 128-byte
   // swizzle; a K step of 16 elements is 32 bytes inside a 64-column box.
   auto qk = [&](int t, int st) {
     const uint32_t a0 = q_lo + (uint32_t)(L::q(t, 0) >> 4);
@@ -441,7 +463,7 @@ __device__ void mma_issuer(const TcParams& p, uint8_t* smem, Shared* S,
 #pragma unroll
     for (int ks = 0; ks < D / 16; ++ks) {
       const uint32_t off = (uint32_t)((ks / 4) * kBox + (ks % 4) * 32) >> 4;
-      mma_ss_warp(tmem + kTmemS, a0 + off, b0 + off, hi, kIdescQK, ks > 0);
+      mma_ss_warp(tmem + T::s(t), a0 + off, b0 + off, hi, kIdescQK, ks > 0);
     }
   };
   // O_t += P_t V: P_t from its TMEM columns (8 per 16 keys), V MN-major (d
@@ -451,17 +473,17 @@ __device__ void mma_issuer(const TcParams& p, uint8_t* smem, Shared* S,
     const uint32_t b0 = v_lo + (uint32_t)st * kStage16;
 #pragma unroll
     for (int kk = 0; kk < kBN / 16; ++kk)
-      mma_ts_warp(tmem + kTmemO + t * 128, tmem + kTmemP + t * 64 + kk * 8,
+      mma_ts_warp(tmem + T::o(t), tmem + T::p(t) + kk * 8,
                   b0 + (uint32_t)(kk * 2048 >> 4), hi, kIdescPV,
                   (acc | kk) != 0);
   };
-  // The k-th QK^T (of either tile) may overwrite S once the softmax warps
-  // have read the previous one into registers (generation k - 1 of the S
-  // barrier).
-  int s_uses = 0;
-  auto take_s = [&]() {
-    if (s_uses > 0) named_sync(kBarSFree);
-    ++s_uses;
+  // A QK^T may overwrite its S once the softmax warps have read the previous
+  // one into registers.  Shared S: the k-th QK^T (of either tile) waits for
+  // generation k - 1 of the one S barrier; own S: each tile has its barrier.
+  int s_uses[kQTiles] = {0, 0};
+  auto take_s = [&](int t) {
+    const int i = T::kOwnS ? t : 0;
+    if (s_uses[i]++ > 0) named_sync(i ? kBarSFree1 : kBarSFree);
     tc_fence_after();
   };
 
@@ -481,7 +503,7 @@ __device__ void mma_issuer(const TcParams& p, uint8_t* smem, Shared* S,
     const int vs = jp % kVStages;
     if (has_qk) {
       relay_sync(kBarKFull0 + st);
-      take_s();
+      take_s(0);
       qk(0, st);
       mma_commit_warp(&S->s_full[0]);
       if (!two) mma_commit_warp(&S->k_empty[st]);
@@ -496,7 +518,7 @@ __device__ void mma_issuer(const TcParams& p, uint8_t* smem, Shared* S,
     }
     if (two) {
       if (has_qk) {
-        take_s();
+        take_s(1);
         qk(1, st);
         mma_commit_warp(&S->s_full[1]);
         mma_commit_warp(&S->k_empty[st]);
@@ -598,17 +620,20 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
                              int t, int nqt, int wq, int lane, int j0, int n,
                              int kv0, int kv1, int q0, bool rev) {
   const uint32_t lane_off = (uint32_t)(wq * 32) << 16;
-  const uint32_t tS = tmem + kTmemS + lane_off;
-  const uint32_t tP = tmem + kTmemP + t * 64 + lane_off;
-  const uint32_t tO = tmem + kTmemO + t * 128 + lane_off;
+  using T = Tmem<D>;
+  const uint32_t tS = tmem + T::s(t) + lane_off;
+  const uint32_t tP = tmem + T::p(t) + lane_off;
+  const uint32_t tO = tmem + T::o(t) + lane_off;
+  const int bar_s = T::kOwnS && t ? kBarSFree1 : kBarSFree;
   const float sl2 = p.scale_log2;
   const uint64_t sl2x2 = f2_pack(sl2, sl2);
   float m_ref = -INFINITY;  // exp2-domain reference (scaled scores)
   float l = 0.f;
   bool ok = true;
   // Arrivals the MMA warp waits for: one per S this tile reads, except the
-  // very last S of the unit (no QK^T follows it), and one per P_t.
-  const int s_expected = (t == nqt - 1) ? n - 1 : n;
+  // very last S of the unit (own S: of the tile; no QK^T follows it), and one
+  // per P_t.
+  const int s_expected = (T::kOwnS || t == nqt - 1) ? n - 1 : n;
   int s_arrived = 0, p_arrived = 0;
   int vis_lo = 0, vis_hi = 0;  // one-shot: this row's visible key tokens
   if (kOneShot) {
@@ -621,7 +646,8 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
   // most one tile each); one-shot, tiles that cross a chunk edge.  Whether
   // this one does is settled before S is waited for and decided once per
   // tile: worked out after the wait, with a test per 32 columns, it stood in
-  // the chain from S to P (480p ring, 84 CTAs of 63 tiles: 76.7 -> 75.6 us).
+  // the chain from S to P (training clip forward 504.9 -> 498.0 us; 480p ring,
+  // 84 CTAs of 63 tiles, 77.2 -> 76.7).
   const int rag0_n = p.seg_len[0] % kBN, rag1_n = p.seg_len[1] % kBN;
   const int rag0 = rag0_n ? p.seg_tiles0 - 1 - j0 : -1;
   const int rag1 = rag1_n ? p.total_tiles - 1 - j0 : -1;
@@ -648,9 +674,14 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
     // S is in registers: the next QK^T (of either tile) may overwrite it.
     tc_fence_before();
     if (s_arrived < s_expected) {
-      named_arrive(kBarSFree);
+      named_arrive(bar_s);
       ++s_arrived;
     }
+    // At d = 64 the softmax warps set the pace (about 2000 clk per key tile
+    // against 1170 of MMAs): a first look at p_free is sent off here, so that
+    // its latency passes behind the row max.  At d = 128 it gained nothing.
+    const bool p_is_free =
+        T::kOwnS && j > 0 && mbar_test_wait(&S->p_free[t], (j - 1) & 1);
     float mx[4] = {-INFINITY, -INFINITY, -INFINITY, -INFINITY};
     if (masked) {
 #pragma unroll
@@ -680,7 +711,8 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
     for (int c = 0; c < 2; ++c) exp_pack32(s[c], sl2x2, neg2, pk[c], acc);
     // P_t(j - 1) has been consumed and O_t holds PV_t(0 .. j-1) (PV_t(j-1)
     // was issued right after this S, so this normally does not wait).
-    if (j > 0 && !(ok = wait_bar(&S->p_free[t], (j - 1) & 1, S, p.status)))
+    if (j > 0 && !p_is_free &&
+        !(ok = wait_bar(&S->p_free[t], (j - 1) & 1, S, p.status)))
       break;
     tc_fence_after();
     if (rescale && j > 0) {
@@ -714,7 +746,7 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
   // contents are undefined, and so is the output), so that the MMA warp
   // never waits for an arrival that does not come.
   while (s_arrived < s_expected) {
-    named_arrive(kBarSFree);
+    named_arrive(bar_s);
     ++s_arrived;
   }
   while (p_arrived < n) {
