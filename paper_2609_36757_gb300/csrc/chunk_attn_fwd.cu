@@ -131,9 +131,11 @@ struct TcParams {
   uint64_t wait_limit_ns;
   int32_t inject_stall;
   // Work split: units of two query tiles, (b, h, pair) with the pair index
-  // fastest; the first units_full run whole, the rest are cut into `split`
-  // key-tile ranges whose partial results go to the workspace.
-  int32_t q_pairs, units_full, split;
+  // fastest, a head's last pair that holds one query tile only (long_pairs)
+  // after all others; the first units_full run whole, the tail_units after
+  // them are cut into `split` key-tile ranges, equal ones or, with cut > 0,
+  // [0, cut) and the rest, whose partial results go to the workspace.
+  int32_t q_pairs, long_pairs, units_full, tail_units, split, cut;
   int32_t sms;  // SM count: CTA index / sms is a CTA's wave
   float* ws;      // partial O: [part][d][kUnitRows]
   float* ws_lse;  // partial log2-domain LSE: [part][kUnitRows]
@@ -198,28 +200,48 @@ __device__ __forceinline__ Work oneshot_work(const TcParams& p) {
   return w;
 }
 
+// Streaming: query pair and (b, h) of a unit; the short units come last.
+__device__ __forceinline__ void unit_coord(const TcParams& p, int unit,
+                                           int& pair, int& bh) {
+  const int n_long = p.long_pairs * p.heads * p.batch;
+  if (unit < n_long) {
+    pair = unit % p.long_pairs;
+    bh = unit / p.long_pairs;
+  } else {
+    pair = p.long_pairs;
+    bh = unit - n_long;
+  }
+}
+
+// The tail's CTAs go range by range, the longer range first: the CTAs that
+// run together then stream the same keys of a head.
 template <bool kOneShot>
 __device__ __forceinline__ Work cta_work(const TcParams& p) {
   if (kOneShot) return oneshot_work(p);
   Work w;
   w.kv0 = w.kv1 = 0;
-  int unit, part = -1, nparts = 1, idx = 0;
-  if ((int)blockIdx.x < p.units_full) {
-    unit = blockIdx.x;
-  } else {
-    const int k = blockIdx.x - p.units_full;
-    unit = p.units_full + k / p.split;
-    idx = k % p.split;
-    part = k;
-    nparts = p.split;
+  w.j0 = 0;
+  w.n = p.total_tiles;
+  int unit = blockIdx.x, part = -1;
+  if (unit >= p.units_full) {
+    const int k = unit - p.units_full;
+    const int u = k % p.tail_units, idx = k / p.tail_units;
+    unit = p.units_full + u;
+    part = u * p.split + idx;
+    if (p.cut > 0) {
+      w.j0 = idx ? p.cut : 0;
+      w.n = idx ? p.total_tiles - p.cut : p.cut;
+    } else {
+      w.j0 = (int)((int64_t)idx * p.total_tiles / p.split);
+      w.n = (int)((int64_t)(idx + 1) * p.total_tiles / p.split) - w.j0;
+    }
   }
-  const int pair = unit % p.q_pairs;
-  w.h = (unit / p.q_pairs) % p.heads;
-  w.b = unit / (p.q_pairs * p.heads);
+  int pair, bh;
+  unit_coord(p, unit, pair, bh);
+  w.h = bh % p.heads;
+  w.b = bh / p.heads;
   w.q0 = pair * kQTiles * kBM;
   w.nqt = (p.q_tokens - w.q0 > kBM) ? 2 : 1;
-  w.j0 = (int)((int64_t)idx * p.total_tiles / nparts);
-  w.n = (int)((int64_t)(idx + 1) * p.total_tiles / nparts) - w.j0;
   w.part = part;
   w.rev = part < 0 && odd_wave(p);
   return w;
@@ -855,10 +877,9 @@ combine_kernel(const __grid_constant__ TcParams p) {
   const int g = threadIdx.x / kMergeRows;
   const int r_unit = blockIdx.y * kMergeRows + r;
   const int col0 = blockIdx.z * kMergeCols + g * kCols;
-  const int unit = p.units_full + ut;
-  const int pair = unit % p.q_pairs;
-  const int h = (unit / p.q_pairs) % p.heads;
-  const int b = unit / (p.q_pairs * p.heads);
+  int pair, bh;
+  unit_coord(p, p.units_full + ut, pair, bh);
+  const int h = bh % p.heads, b = bh / p.heads;
   const int row0 = pair * kQTiles * kBM + blockIdx.y * kMergeRows;
   if (row0 >= p.q_tokens) return;  // the whole block is past the chunk end
   const int k0 = ut * p.split;
@@ -922,6 +943,89 @@ combine_kernel(const __grid_constant__ TcParams p) {
     if (row < p.q_tokens && in_bounds(x, p.o_elems - 7, p.status))
       *reinterpret_cast<uint4*>(p.o + x) =
           *reinterpret_cast<const uint4*>(&tile[rr][piece * 8]);
+  }
+}
+
+// The same merge for at most kFewParts parts per unit: many units then,
+// and little to do for each, so a thread takes four rows x eight columns with
+// 16-byte loads and writes each row's 16 bytes straight out, and a CTA takes
+// all 256 rows of a unit x 32 columns.  (Blocks of 32 rows with 4-byte loads,
+// as above: 2688 of them for 84 units, 11.1 us against 8.3; 56 units, 12.8
+// against 7.8.  With fewer blocks than SMs this form loses: 4 units, 5.4 us
+// against 4.6.)
+constexpr int kFewParts = 4;
+constexpr int kFewCols = 8;  // columns per thread
+constexpr int kFewThreads = kUnitRows / 4 * (kMergeCols / kFewCols);  // 256
+
+template <int D>
+__global__ void __launch_bounds__(kFewThreads)
+combine_few_kernel(const __grid_constant__ TcParams p) {
+  pdl_trigger();
+  pdl_wait();  // the partial results of the attention kernel are complete
+  const int ut = blockIdx.x;
+  const int r0 = threadIdx.x % (kUnitRows / 4) * 4;
+  const int col0 = blockIdx.y * kMergeCols + threadIdx.x / (kUnitRows / 4) * kFewCols;
+  const int parts = p.split;
+  int pair, bh;
+  unit_coord(p, p.units_full + ut, pair, bh);
+  const int row0 = pair * kQTiles * kBM + r0;
+  if (row0 >= p.q_tokens) return;
+  const int k0 = ut * parts;
+  // every part this block reads lies in the workspace
+  if (!in_bounds(k0 + parts - 1, p.ws_parts, p.status)) return;
+  const float* lse = p.ws_lse + (size_t)k0 * kUnitRows + r0;
+  float w[kFewParts][4], m[4], wsum[4] = {0.f, 0.f, 0.f, 0.f};
+#pragma unroll
+  for (int r = 0; r < 4; ++r) m[r] = -INFINITY;
+#pragma unroll
+  for (int u = 0; u < kFewParts; ++u) {
+    float4 l = make_float4(-INFINITY, -INFINITY, -INFINITY, -INFINITY);
+    if (u < parts)
+      l = *reinterpret_cast<const float4*>(lse + (size_t)u * kUnitRows);
+    w[u][0] = l.x, w[u][1] = l.y, w[u][2] = l.z, w[u][3] = l.w;
+#pragma unroll
+    for (int r = 0; r < 4; ++r) m[r] = fmaxf(m[r], w[u][r]);
+  }
+#pragma unroll
+  for (int u = 0; u < kFewParts; ++u)
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+      w[u][r] = ex2(w[u][r] - m[r]);  // 0 for the missing parts
+      wsum[r] += w[u][r];
+    }
+  float acc[kFewCols][4] = {};
+  const float* src = p.ws + ((size_t)k0 * D + col0) * kUnitRows + r0;
+#pragma unroll
+  for (int u = 0; u < kFewParts; ++u) {
+    if (u >= parts) break;
+#pragma unroll
+    for (int x = 0; x < kFewCols; ++x) {
+      const float4 v = *reinterpret_cast<const float4*>(
+          src + ((size_t)u * D + x) * kUnitRows);
+      acc[x][0] = fmaf(w[u][0], v.x, acc[x][0]);
+      acc[x][1] = fmaf(w[u][1], v.y, acc[x][1]);
+      acc[x][2] = fmaf(w[u][2], v.z, acc[x][2]);
+      acc[x][3] = fmaf(w[u][3], v.w, acc[x][3]);
+    }
+  }
+  const int h = bh % p.heads, b = bh / p.heads;
+#pragma unroll
+  for (int r = 0; r < 4; ++r) {
+    const int row = row0 + r;
+    if (row >= p.q_tokens) return;
+    const float inv = 1.f / wsum[r];
+    const int64_t x = (int64_t)b * p.o_str.batch + (int64_t)row * p.o_str.token +
+                      (int64_t)h * p.o_str.head + col0;
+    if (in_bounds(x, p.o_elems - 7, p.status))
+      *reinterpret_cast<uint4*>(p.o + x) =
+          make_uint4(pack_bf16(acc[0][r] * inv, acc[1][r] * inv),
+                     pack_bf16(acc[2][r] * inv, acc[3][r] * inv),
+                     pack_bf16(acc[4][r] * inv, acc[5][r] * inv),
+                     pack_bf16(acc[6][r] * inv, acc[7][r] * inv));
+    const int64_t lse_i = ((int64_t)b * p.heads + h) * p.q_tokens + row;
+    if (col0 == 0 && p.lse != nullptr &&
+        in_bounds(lse_i, (int64_t)p.batch * p.heads * p.q_tokens, p.status))
+      p.lse[lse_i] = (m[r] + __log2f(wsum[r])) * 0.6931471805599453f;
   }
 }
 
@@ -1005,24 +1109,52 @@ int sm_count() {
   return n > 0 ? n : 1;
 }
 
-// Units of two query tiles: whole waves of units run whole, and the units of
-// a last partial wave are cut along the keys so that every SM has work (at
-// least kMinTilesPerPart key tiles per part, at most max_parts parts).
-void split_units(int units, int tiles, int sms, int max_parts, int* units_full,
-                 int* split) {
+// How a launch's units of two query tiles are spread over the SMs.
+struct Split {
+  int units_full;  // units that run whole, a CTA each
+  int split;       // parts of each unit after those
+  int cut;         // 0: equal parts; else the key tiles of the first of two
+};
+
+// Whole waves of units run whole; the units of a last partial wave are cut
+// along the keys where that ends sooner.  Counted in key tiles of two query
+// tiles (about 1.1 us at d = 128): a CTA costs its tiles and kCtaCost (set-up,
+// first loads, filling and draining the pipeline, epilogue: 10.8k clk against
+// 2240 per tile), the merge of the parts kMergeCost (its launch, here and on
+// the host, and its fixed time) and 1 / kPartsPerTile for each.  Equal parts may take more than one round on the SMs.  Where most of
+// the SMs have a unit already, two unequal parts: one for a CTA on each of
+// `rem` SMs, the others go round the rest, at most q on one SM, and the cut
+// lies where both end together.  (Equal parts in one round at most left 68 of
+// 152 SMs idle for a 480p frame, 84 units of 63 tiles:
+// 76.8 us, now 65.9 with the merge.)
+Split split_units(int units, int tiles, int sms, int max_parts) {
+  constexpr double kCtaCost = 5.0, kMergeCost = 6.0, kPartsPerTile = 40.0;
   const int rem = units % sms;
-  int s = 1;
-  if (rem > 0) {
-    s = std::min(sms / rem, tiles / kMinTilesPerPart);
-    s = std::min(s, std::min(kMaxParts, max_parts) / rem);
+  Split best = {units, 1, 0};
+  if (rem == 0) return best;
+  double best_cost = tiles + kCtaCost;
+  auto merge = [&](int s) { return kMergeCost + rem * s / kPartsPerTile; };
+  for (int s = 2; s * kMinTilesPerPart <= tiles && rem * s <= max_parts; ++s) {
+    const int rounds = (rem * s + sms - 1) / sms;
+    const double cost = rounds * ((tiles + s - 1) / s + kCtaCost) + merge(s);
+    if (cost < best_cost) {
+      best_cost = cost;
+      best = {units - rem, s, 0};
+    }
   }
-  if (s >= 2) {
-    *units_full = units - rem;
-    *split = s;
-  } else {
-    *units_full = units;
-    *split = 1;
+  if (2 * rem > sms && 2 * rem <= max_parts) {
+    const int q = (rem + sms - rem - 1) / (sms - rem);
+    const int cut = (int)ceil((q * (tiles + kCtaCost) - kCtaCost) / (1 + q));
+    if (cut >= kMinTilesPerPart && tiles - cut >= kMinTilesPerPart &&
+        cut + kCtaCost + merge(2) < best_cost)
+      best = {units - rem, 2, cut};
   }
+  return best;
+}
+
+// Query pairs of a head with rows in both of their tiles.
+int long_pairs(int q_tokens) {
+  return (q_tokens + kBM - 1) / (kQTiles * kBM);
 }
 
 int total_tiles(const AttnParams& a) {
@@ -1093,10 +1225,14 @@ cudaError_t launch_d(const AttnParams& a, cudaStream_t stream, int* launches) {
   p.q_pairs = (a.q_tokens + kQTiles * kBM - 1) / (kQTiles * kBM);
   const int units = p.q_pairs * a.heads * a.batch;
   p.sms = sm_count();
-  split_units(units, tiles, p.sms, a.workspace_parts, &p.units_full,
-              &p.split);
+  p.long_pairs = long_pairs(a.q_tokens);
+  const Split sp = split_units(units, tiles, p.sms, split_parts(D));
+  p.units_full = sp.units_full;
+  p.tail_units = units - sp.units_full;
+  p.split = sp.split;
+  p.cut = sp.cut;
   p.ws_lse = p.ws + (size_t)a.workspace_parts * D * kUnitRows;
-  const int grid = p.units_full + (units - p.units_full) * p.split;
+  const int grid = p.units_full + p.tail_units * p.split;
   const int smem = Layout<D>::bytes;
   cudaError_t e = cudaFuncSetAttribute(
       chunk_attn_tc_kernel<D, false>, cudaFuncAttributeMaxDynamicSharedMemorySize,
@@ -1107,10 +1243,15 @@ cudaError_t launch_d(const AttnParams& a, cudaStream_t stream, int* launches) {
   if (e != cudaSuccess) return e;
   *launches = 1;
   if (p.split > 1) {
-    e = launch_pdl(combine_kernel<D>,
-                   dim3(units - p.units_full, kUnitRows / kMergeRows,
-                        D / kMergeCols),
-                   dim3(kMergeThreads), 0, stream, p);
+    const bool few =
+        p.split <= kFewParts && p.tail_units * (D / kMergeCols) >= p.sms;
+    e = few ? launch_pdl(combine_few_kernel<D>,
+                         dim3(p.tail_units, D / kMergeCols),
+                         dim3(kFewThreads), 0, stream, p)
+            : launch_pdl(combine_kernel<D>,
+                         dim3(p.tail_units, kUnitRows / kMergeRows,
+                              D / kMergeCols),
+                         dim3(kMergeThreads), 0, stream, p);
     if (e != cudaSuccess) return e;
     *launches = 2;
   }
@@ -1177,9 +1318,9 @@ cudaError_t launch_blockcausal_attn(const OneShotParams& p, cudaStream_t stream)
 int chunk_attn_parts(const AttnParams& a) {
   const int pairs = (a.q_tokens + kQTiles * kBM - 1) / (kQTiles * kBM);
   const int units = pairs * a.heads * a.batch;
-  int full = 0, split = 1;
-  split_units(units, total_tiles(a), sm_count(), kMaxParts, &full, &split);
-  return split > 1 ? (units - full) * split : 0;
+  const Split sp =
+      split_units(units, total_tiles(a), sm_count(), split_parts(a.head_dim));
+  return sp.split > 1 ? (units - sp.units_full) * sp.split : 0;
 }
 
 cudaError_t launch_chunk_attn(const AttnParams& p, cudaStream_t stream,

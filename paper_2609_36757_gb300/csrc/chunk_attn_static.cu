@@ -30,7 +30,7 @@ namespace {
 
 // 24 MiB: room for 190 partial results at d = 128 (378 at d = 64); a GB300
 // launch uses at most one per SM (152).
-constexpr size_t kScratchBytes = size_t(24) << 20;
+constexpr size_t kScratchBytes = fastvr::kStaticScratchBytes;
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
 
@@ -150,8 +150,7 @@ extern "C" fastvr_status_t fastvr_chunk_attn_fwd_static(
   // them than fit is refused rather than run with a different split.  The
   // array keeps the last call's contents, which needs no clearing: every
   // partial result is written before it is read.
-  const size_t part_bytes = (size_t)fastvr::kUnitRows * (d + 1) * sizeof(float);
-  const int capacity = (int)(kScratchBytes / part_bytes);
+  const int capacity = (int)(kScratchBytes / fastvr::part_bytes(d));
   if (fastvr::chunk_attn_parts(a) > capacity) return FASTVR_ERR_CAPACITY;
   a.workspace = reinterpret_cast<float*>(scratch);
   a.workspace_parts = capacity;

@@ -19,6 +19,18 @@ constexpr int kMaxSegments = 2;
 // results of 256 query rows, each d fp32 outputs plus one log-sum-exp.
 constexpr int kMaxParts = 256;
 constexpr int kUnitRows = 256;
+// Scratch array of the allocation-free entry point, and the most partial
+// results that any launch leaves: what fits both it and the plan's workspace,
+// so that the two entry points split the same work the same way.
+constexpr size_t kStaticScratchBytes = size_t(24) << 20;
+constexpr size_t part_bytes(int head_dim) {
+  return (size_t)kUnitRows * (head_dim + 1) * sizeof(float);
+}
+constexpr int split_parts(int head_dim) {
+  return kStaticScratchBytes / part_bytes(head_dim) < (size_t)kMaxParts
+             ? (int)(kStaticScratchBytes / part_bytes(head_dim))
+             : kMaxParts;
+}
 inline size_t workspace_bytes(int head_dim) {
   return (size_t)kMaxParts * kUnitRows * (head_dim + 1) * sizeof(float);
 }

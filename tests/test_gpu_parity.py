@@ -114,6 +114,33 @@ def test_random_small_stream_every_element(w):
     err.check()
 
 
+# How a launch's units of 256 query rows are spread over 152 SMs: units cut in
+# two unequal parts, short units (at most 128 rows) behind the others, both
+# merges.  Sampled rows against the oracle, with the tolerances of every other
+# stream.
+SPLITS = [
+    # 85 units of up to 44 tiles: two unequal parts each
+    WL.custom("unequal-parts", batch=1, heads=17, head_dim=64,
+              tokens_per_frame=1120, frames_per_chunk=1, num_chunks=5, seed=81),
+    # 165 units: 132 long and 20 short ones whole, then 13 short ones in parts
+    WL.custom("short-tail", batch=1, heads=33, head_dim=128,
+              tokens_per_frame=1100, frames_per_chunk=1, num_chunks=3, seed=82),
+    # every unit short, more than one wave, a wrapped ring with a ragged end
+    WL.custom("all-short", batch=2, heads=80, head_dim=64,
+              tokens_per_frame=100, frames_per_chunk=1, num_chunks=9,
+              window_chunks=6, seed=83),
+    # 152 units: no tail at all; and one tile per unit
+    WL.custom("whole-wave", batch=2, heads=76, head_dim=128,
+              tokens_per_frame=70, frames_per_chunk=2, num_chunks=3,
+              last_chunk_frames=1, seed=84),
+]
+
+
+@pytest.mark.parametrize("w", SPLITS, ids=lambda w: w.name)
+def test_work_split_shapes(w):
+    run_stream(w, rows_per_chunk=48).check()
+
+
 @pytest.mark.parametrize("w", SMALL[:3], ids=lambda w: w.name)
 def test_streamed_gpu_equals_oneshot_oracle(FV, w):
     att = FV.StreamingAttention(FV.config_from_workload(w))
