@@ -1193,16 +1193,20 @@ cudaError_t launch_d(const AttnParams& a, cudaStream_t stream, int* launches) {
     return cudaErrorInvalidValue;
   int tiles = 0;
   for (int s = 0; s < kMaxSegments; ++s) {
-    const int src = s < a.num_segments ? s : 0;
+    if (s >= a.num_segments) {  // never read: seg_len stays 0
+      p.k_map[s] = p.k_map[0];
+      p.v_map[s] = p.v_map[0];
+      continue;
+    }
     // The map ends where the segment ends: keys past it read as zeros.
-    const int64_t end = a.seg_start[src] + a.seg_len[src];
+    const int64_t end = a.seg_start[s] + a.seg_len[s];
     if (!make_map(&p.k_map[s], a.k, D, end, a.heads, a.batch,
                   a.kv_str.token * es, a.kv_str.head * es, a.kv_str.batch * es) ||
         !make_map(&p.v_map[s], a.v, D, end, a.heads, a.batch,
                   a.kv_str.token * es, a.kv_str.head * es, a.kv_str.batch * es))
       return cudaErrorInvalidValue;
-    p.seg_start[s] = (int32_t)a.seg_start[src];
-    p.seg_len[s] = s < a.num_segments ? a.seg_len[s] : 0;
+    p.seg_start[s] = (int32_t)a.seg_start[s];
+    p.seg_len[s] = a.seg_len[s];
     const int t = (p.seg_len[s] + kBN - 1) / kBN;
     if (s == 0) p.seg_tiles0 = t;
     tiles += t;

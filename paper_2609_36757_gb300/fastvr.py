@@ -16,6 +16,11 @@ import ctypes
 import os
 from typing import Optional, Tuple
 
+try:  # only the torch conveniences below need it
+    import torch
+except ImportError:
+    torch = None
+
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libfastvr_attn.so")
 # The same library with device-side index checks (FASTVR_BOUNDS_CHECK).
@@ -116,6 +121,23 @@ def _check(status: int, where: str) -> None:
         raise FastVRError(status, where)
 
 
+def _current_stream() -> int:
+    """cudaStream_t of torch's current stream on the current device.  A small
+    call is bound by its host time, and building a torch.cuda.Stream object
+    for its handle took 2.8 us of it; the raw handle takes 0.1."""
+    return _raw_stream(_current_device())
+
+
+def _stream_handle(_device: int) -> int:
+    return torch.cuda.current_stream().cuda_stream
+
+
+_raw_stream = getattr(getattr(torch, "_C", None), "_cuda_getCurrentRawStream",
+                      _stream_handle)
+_current_device = getattr(getattr(torch, "_C", None), "_cuda_getDevice",
+                          lambda: 0)
+
+
 # ------------------------------------------------------------ C-named calls
 def fastvr_status_string(status: int) -> str:
     return lib.fastvr_status_string(status).decode()
@@ -204,13 +226,14 @@ def blockcausal_attention(cfg: fastvr_attn_config_t, q, k, v,
                           want_lse: bool = False):
     """Torch convenience for fastvr_blockcausal_attn_fwd: q, k, v contiguous
     bfloat16 CUDA tensors [B, L, H, d]; runs on the current stream."""
-    import torch
+    bf16 = torch.bfloat16
     for t in (q, k, v):
-        if t.dtype != torch.bfloat16 or not t.is_cuda or not t.is_contiguous():
+        if t.dtype != bf16 or not t.is_cuda or not t.is_contiguous():
             raise ValueError("q, k, v must be contiguous bfloat16 CUDA tensors")
-    if not (q.shape == k.shape == v.shape):
+    shape = q.shape
+    if not (shape == k.shape == v.shape):
         raise ValueError("q, k, v differ in shape")
-    B, L, H, d = q.shape
+    B, L, H, d = shape
     if (B, H, d) != (cfg.batch, cfg.heads, cfg.head_dim) or \
             L % cfg.tokens_per_frame:
         raise ValueError(f"q has shape {tuple(q.shape)}")
@@ -220,7 +243,7 @@ def blockcausal_attention(cfg: fastvr_attn_config_t, q, k, v,
     fastvr_blockcausal_attn_fwd(cfg, L // cfg.tokens_per_frame, q.data_ptr(),
                                 k.data_ptr(), v.data_ptr(), out.data_ptr(),
                                 0 if lse is None else lse.data_ptr(),
-                                torch.cuda.current_stream().cuda_stream)
+                                _current_stream())
     return (out, lse) if want_lse else out
 
 
@@ -245,7 +268,6 @@ def blockcausal_attention_bwd(cfg: fastvr_attn_config_t, q, k, v, out, dout,
     """Torch convenience for fastvr_blockcausal_attn_bwd: bfloat16 CUDA
     tensors [B, L, H, d] and the forward's float32 lse [B, H, L]; returns
     (dq, dk, dv).  The scratch is allocated with torch."""
-    import torch
     L = q.shape[1]
     frames = L // cfg.tokens_per_frame
     nbytes = fastvr_blockcausal_bwd_scratch_bytes(cfg, frames)
@@ -254,8 +276,7 @@ def blockcausal_attention_bwd(cfg: fastvr_attn_config_t, q, k, v, out, dout,
     fastvr_blockcausal_attn_bwd(
         cfg, frames, q.data_ptr(), k.data_ptr(), v.data_ptr(), out.data_ptr(),
         dout.data_ptr(), lse.data_ptr(), dq.data_ptr(), dk.data_ptr(),
-        dv.data_ptr(), scratch.data_ptr(), nbytes,
-        torch.cuda.current_stream().cuda_stream)
+        dv.data_ptr(), scratch.data_ptr(), nbytes, _current_stream())
     return dq, dk, dv
 
 
@@ -269,9 +290,8 @@ def one_step_update(z_lq, v, sigma: float, out=None):
     """Torch convenience: z_lq bfloat16 or float32, v bfloat16, same shape,
     contiguous CUDA tensors; returns z_lq - sigma * v (in place when
     out is z_lq)."""
-    import torch
-    if v.dtype != torch.bfloat16 or z_lq.dtype not in (torch.bfloat16,
-                                                       torch.float32):
+    zt = z_lq.dtype
+    if v.dtype != torch.bfloat16 or zt not in (torch.bfloat16, torch.float32):
         raise ValueError("z_lq must be bfloat16 or float32 and v bfloat16")
     if z_lq.shape != v.shape or not (z_lq.is_contiguous() and v.is_contiguous()):
         raise ValueError("z_lq and v must be contiguous and of one shape")
@@ -279,8 +299,8 @@ def one_step_update(z_lq, v, sigma: float, out=None):
         out = torch.empty_like(z_lq)
     fastvr_one_step_update(z_lq.data_ptr(), v.data_ptr(), out.data_ptr(),
                            z_lq.numel(), sigma,
-                           0 if z_lq.dtype == torch.bfloat16 else 1,
-                           torch.cuda.current_stream().cuda_stream)
+                           0 if zt == torch.bfloat16 else 1,
+                           _current_stream())
     return out
 
 
@@ -334,7 +354,6 @@ class StreamingAttention:
     (contiguous, token-major) and enqueue on the current CUDA stream."""
 
     def __init__(self, cfg: fastvr_attn_config_t, device=None):
-        import torch
         self.cfg = cfg
         self.nbytes = fastvr_kv_cache_bytes(cfg)
         self.cache = torch.empty(self.nbytes, dtype=torch.uint8,
@@ -348,7 +367,6 @@ class StreamingAttention:
             self.plan = None
 
     def _check_chunk(self, t, name: str) -> int:
-        import torch
         c = self.cfg
         if t.dtype != torch.bfloat16 or not t.is_cuda or not t.is_contiguous():
             raise ValueError(f"{name} must be a contiguous bfloat16 CUDA tensor")
@@ -359,8 +377,7 @@ class StreamingAttention:
 
     @staticmethod
     def _stream() -> int:
-        import torch
-        return torch.cuda.current_stream().cuda_stream
+        return _current_stream()
 
     def append(self, k, v) -> None:
         frames = self._check_chunk(k, "k")
@@ -371,7 +388,6 @@ class StreamingAttention:
 
     def forward(self, q, out=None, lse: Optional[object] = None,
                 want_lse: bool = False):
-        import torch
         self._check_chunk(q, "q")
         if out is None:
             out = torch.empty_like(q)
