@@ -68,6 +68,12 @@ constexpr int kBarDS = 2;
 constexpr int kBarRing0 = 3;  // + stage, up to kMaxStages
 constexpr int kBarRing1 = 6;  // + stage, up to kStages1
 constexpr int kBarStaged = 8;  // the compute warps' output tiles are staged
+// The dQ kernel hands dS over through two barriers in turn (kBarDS, kBarDSOdd):
+// its next S and dP do not wait for dS, so a compute warp can be done with the
+// next dS while another has yet to arrive for this one, and on one barrier its
+// second arrival would stand in for the other's first.  It cannot be two ahead:
+// the S after that follows the MMA warp's wait for this dS.
+constexpr int kBarDSOdd = 9;
 constexpr int kComputeHandoff = 9 * 32;
 constexpr int kRelayHandoff = 2 * 32;
 constexpr uint32_t kTmemCols = 512;
@@ -858,7 +864,10 @@ dq_kernel(const __grid_constant__ BwdParams p) {
         mma_commit_warp(&S->dp_ready[(j + 1) & 1]);
         mma_commit_warp(&S->empty[1][v_stn]);  // V_{j+1} read for the last time
       }
-      compute_sync(kBarDS);
+      if (j & 1)
+        compute_sync(kBarDSOdd);
+      else
+        compute_sync(kBarDS);
       tc_fence_after();
       mma_tn<D>(sbase, tmem, 256, dq_dp_col(j), L::ring(k_st, 0, 0), j > 0);  // dQ
       mma_commit_warp(&S->empty[0][k_st]);  // K_j read for the last time
@@ -902,7 +911,9 @@ dq_kernel(const __grid_constant__ BwdParams p) {
       const int lo_m = in_range ? lo : 64, hi_m = in_range ? hi : 0;
       uint32_t x0[32], x1[32], pb0[16], pb1[16], pk[16];
       // phase 1 (overlaps the dP MMAs): P (bf16 pairs) in registers; S is
-      // then free for the next tile
+      // then free for the next tile (released as soon as it has been read, the
+      // next S and dP ran beside P and cost it more than they gained: crop
+      // training step 141.7 -> 143.8 us)
       tmem_ld32(row_t + cs, x0);
       tmem_ld32(row_t + cs + 32, x1);
       tmem_wait_ld();
@@ -930,14 +941,18 @@ dq_kernel(const __grid_constant__ BwdParams p) {
       tmem_st16(row_t + cp + 16, pk);
       tmem_wait_st();
       tc_fence_before();
-      compute_arrive(kBarDS);
+      if (j & 1)
+        compute_arrive(kBarDSOdd);
+      else
+        compute_arrive(kBarDS);
       ++ds_arr;
     }
     // After a failed wait the remaining hand-offs are still made (with
     // undefined contents), so that the MMA warp never waits for an arrival
     // that does not come.
     for (; p_arr < n; ++p_arr) compute_arrive(kBarP);
-    for (; ds_arr < n; ++ds_arr) compute_arrive(kBarDS);
+    for (; ds_arr < n; ++ds_arr)
+      compute_arrive(ds_arr & 1 ? kBarDSOdd : kBarDS);
     // dQ is staged in the first K stage (free once o_full has completed)
     // and leaves as TMA stores; rows past the sequence are not written.
     uint8_t* const tiles[1] = {smem + L::ring(0, 0, 0)};
