@@ -167,8 +167,8 @@ FASTVR_API fastvr_status_t fastvr_plan_visible(fastvr_plan_t plan, int32_t* num_
  * chunk).  q, k, v: bfloat16 [B, L, H, d] token-major with L = num_frames *
  * N; out bfloat16 [B, L, H, d]; lse nullable, float32 [B, H, L].  Frame f
  * belongs to chunk f / k; a ragged final chunk is simply shorter.  Each
- * block of 256 query rows reads only the keys its rows can see (invisible
- * chunks are never loaded); rows that straddle a chunk boundary are masked
+ * block of 256 query rows (128 where the launch has few) reads only the keys
+ * its rows can see (invisible chunks are never loaded); rows that straddle a chunk boundary are masked
  * element-wise.  No plan, no cache and no scratch memory are involved; a
  * bounded-wait timeout leaves out undefined and is reported by
  * fastvr_get_device_status.  The result

@@ -136,6 +136,7 @@ struct TcParams {
   // them are cut into `split` key-tile ranges, equal ones or, with cut > 0,
   // [0, cut) and the rest, whose partial results go to the workspace.
   int32_t q_pairs, long_pairs, units_full, tail_units, split, cut;
+  int32_t unit_rows;  // query rows of a unit: two tiles, or one (few units)
   int32_t sms;  // SM count: CTA index / sms is a CTA's wave
   float* ws;      // partial O: [part][d][kUnitRows]
   float* ws_lse;  // partial log2-domain LSE: [part][kUnitRows]
@@ -186,10 +187,11 @@ __device__ __forceinline__ Work oneshot_work(const TcParams& p) {
   const int pair = p.q_pairs - 1 - blk * kOneShotBlock - x % in_blk;
   w.h = bh % p.heads;
   w.b = bh / p.heads;
-  w.q0 = pair * kQTiles * kBM;
-  w.nqt = (p.q_tokens - w.q0 > kBM) ? 2 : 1;
+  w.q0 = pair * p.unit_rows;
+  const int rows = min(p.unit_rows, p.q_tokens - w.q0);
+  w.nqt = rows > kBM ? 2 : 1;
   const int c_lo = w.q0 / p.chunk_tokens;
-  const int c_hi = min(w.q0 + kQTiles * kBM, p.q_tokens) - 1;
+  const int c_hi = w.q0 + rows - 1;
   const int chunk_hi = c_hi / p.chunk_tokens;
   w.kv0 = p.window < 0 ? 0 : max(0, c_lo - p.window) * p.chunk_tokens;
   w.kv1 = min((chunk_hi + 1) * p.chunk_tokens, p.seq_tokens);
@@ -240,8 +242,8 @@ __device__ __forceinline__ Work cta_work(const TcParams& p) {
   unit_coord(p, unit, pair, bh);
   w.h = bh % p.heads;
   w.b = bh / p.heads;
-  w.q0 = pair * kQTiles * kBM;
-  w.nqt = (p.q_tokens - w.q0 > kBM) ? 2 : 1;
+  w.q0 = pair * p.unit_rows;
+  w.nqt = min(p.unit_rows, p.q_tokens - w.q0) > kBM ? 2 : 1;
   w.part = part;
   w.rev = part < 0 && odd_wave(p);
   return w;
@@ -1114,7 +1116,12 @@ struct Split {
   int units_full;  // units that run whole, a CTA each
   int split;       // parts of each unit after those
   int cut;         // 0: equal parts; else the key tiles of the first of two
+  int unit_rows;   // query rows of a unit
 };
+
+// Time of a key tile with one query tile, in units of one with two: its QK^T,
+// softmax and PV follow one another (480p, 25 to 199 key tiles: 0.72-0.78).
+constexpr double kOneTileCost = 0.75;
 
 // Whole waves of units run whole; the units of a last partial wave are cut
 // along the keys where that ends sooner.  Counted in key tiles of two query
@@ -1127,10 +1134,15 @@ struct Split {
 // lies where both end together.  (Equal parts in one round at most left 68 of
 // 152 SMs idle for a 480p frame, 84 units of 63 tiles:
 // 76.8 us, now 65.9 with the merge.)
-Split split_units(int units, int tiles, int sms, int max_parts) {
+//
+// Where twice the units still fit the SMs, units of one query tile are the
+// other way to use more of them, and cost no merge (chunk of 600 queries x 2400
+// keys, 12 heads, d = 64: 26.4 -> 21.2 us).
+Split split_units(int units, int one_tile_units, int tiles, int sms,
+                  int max_parts) {
   constexpr double kCtaCost = 5.0, kMergeCost = 6.0, kPartsPerTile = 40.0;
   const int rem = units % sms;
-  Split best = {units, 1, 0};
+  Split best = {units, 1, 0, kUnitRows};
   if (rem == 0) return best;
   double best_cost = tiles + kCtaCost;
   auto merge = [&](int s) { return kMergeCost + rem * s / kPartsPerTile; };
@@ -1139,17 +1151,27 @@ Split split_units(int units, int tiles, int sms, int max_parts) {
     const double cost = rounds * ((tiles + s - 1) / s + kCtaCost) + merge(s);
     if (cost < best_cost) {
       best_cost = cost;
-      best = {units - rem, s, 0};
+      best = {units - rem, s, 0, kUnitRows};
     }
   }
   if (2 * rem > sms && 2 * rem <= max_parts) {
     const int q = (rem + sms - rem - 1) / (sms - rem);
     const int cut = (int)ceil((q * (tiles + kCtaCost) - kCtaCost) / (1 + q));
     if (cut >= kMinTilesPerPart && tiles - cut >= kMinTilesPerPart &&
-        cut + kCtaCost + merge(2) < best_cost)
-      best = {units - rem, 2, cut};
+        cut + kCtaCost + merge(2) < best_cost) {
+      best_cost = cut + kCtaCost + merge(2);
+      best = {units - rem, 2, cut, kUnitRows};
+    }
   }
+  if (one_tile_units > units && one_tile_units <= sms &&
+      kOneTileCost * tiles + kCtaCost < best_cost)
+    best = {one_tile_units, 1, 0, kBM};
   return best;
+}
+
+// Units of a head.
+int units_of(int q_tokens, int unit_rows) {
+  return (q_tokens + unit_rows - 1) / unit_rows;
 }
 
 // Query pairs of a head with rows in both of their tiles.
@@ -1226,13 +1248,17 @@ cudaError_t launch_d(const AttnParams& a, cudaStream_t stream, int* launches) {
   p.inject_stall = a.inject_stall;
   p.ws = a.workspace;
 
-  p.q_pairs = (a.q_tokens + kQTiles * kBM - 1) / (kQTiles * kBM);
-  const int units = p.q_pairs * a.heads * a.batch;
+  const int bh = a.heads * a.batch;
+  const int units = units_of(a.q_tokens, kUnitRows) * bh;
   p.sms = sm_count();
-  p.long_pairs = long_pairs(a.q_tokens);
-  const Split sp = split_units(units, tiles, p.sms, split_parts(D));
+  const Split sp = split_units(units, units_of(a.q_tokens, kBM) * bh, tiles,
+                               p.sms, split_parts(D));
+  p.unit_rows = sp.unit_rows;
+  p.q_pairs = units_of(a.q_tokens, sp.unit_rows);
+  p.long_pairs =
+      sp.unit_rows == kUnitRows ? long_pairs(a.q_tokens) : p.q_pairs;
   p.units_full = sp.units_full;
-  p.tail_units = units - sp.units_full;
+  p.tail_units = p.q_pairs * bh - sp.units_full;
   p.split = sp.split;
   p.cut = sp.cut;
   p.ws_lse = p.ws + (size_t)a.workspace_parts * D * kUnitRows;
@@ -1297,9 +1323,15 @@ cudaError_t launch_oneshot_d(const OneShotParams& a, cudaStream_t stream) {
   p.seq_tokens = a.seq_tokens;
   p.chunk_tokens = a.chunk_tokens;
   p.window = a.window;
-  p.q_pairs = (a.seq_tokens + kQTiles * kBM - 1) / (kQTiles * kBM);
-  p.split = 1;
   p.sms = sm_count();
+  // Units of one query tile where twice the units still fit the SMs: 9000
+  // tokens, 2 heads, no window: 98.1 -> 75.2 us; 2400 tokens, 8 heads, W = 1:
+  // 32.0 -> 23.7.  (With more units they would take a second round.)
+  p.unit_rows = units_of(a.seq_tokens, kBM) * a.heads * a.batch <= p.sms
+                    ? kBM
+                    : kUnitRows;
+  p.q_pairs = units_of(a.seq_tokens, p.unit_rows);
+  p.split = 1;
   const int grid = p.q_pairs * a.heads * a.batch;
   p.units_full = grid;
   const int smem = Layout<D>::bytes;
@@ -1320,10 +1352,11 @@ cudaError_t launch_blockcausal_attn(const OneShotParams& p, cudaStream_t stream)
 }
 
 int chunk_attn_parts(const AttnParams& a) {
-  const int pairs = (a.q_tokens + kQTiles * kBM - 1) / (kQTiles * kBM);
-  const int units = pairs * a.heads * a.batch;
-  const Split sp =
-      split_units(units, total_tiles(a), sm_count(), split_parts(a.head_dim));
+  const int bh = a.heads * a.batch;
+  const int units = units_of(a.q_tokens, kUnitRows) * bh;
+  const Split sp = split_units(units, units_of(a.q_tokens, kBM) * bh,
+                               total_tiles(a), sm_count(),
+                               split_parts(a.head_dim));
   return sp.split > 1 ? (units - sp.units_full) * sp.split : 0;
 }
 

@@ -48,6 +48,14 @@ CASES = [
     # k N = 128: query tiles and chunks align
     WL.custom("aligned", batch=1, heads=2, head_dim=128, tokens_per_frame=64,
               frames_per_chunk=2, num_chunks=9, seed=66),
+    # the cases above have so few units that each takes one query tile; here
+    # units of two tiles straddle chunk boundaries, in one wave and in two
+    WL.custom("two-tiles-d128", batch=1, heads=32, head_dim=128,
+              tokens_per_frame=150, frames_per_chunk=2, num_chunks=3,
+              window_chunks=1, last_chunk_frames=1, seed=69),
+    WL.custom("two-tiles-d64", batch=2, heads=24, head_dim=64,
+              tokens_per_frame=170, frames_per_chunk=1, num_chunks=5,
+              seed=70),
 ]
 
 
