@@ -480,7 +480,7 @@ __device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v 
 // nearest integer (x + 1.5 * 2^23 rounds it into the low mantissa bits) and
 // f in [-0.5, 0.5]; 2^f by a degree-3 polynomial (a relative-error minimax
 // fit on [-0.5, 0.5], at most 7.5e-5 relative error in fp32: far below the
-// 2^-9 of the bf16 P it feeds), then n added to its exponent field.  x is
+// 2^-9 of the bf16 P or dS it feeds), then n added to its exponent field.  x is
 // first clamped to >= -126 so that the exponent cannot wrap (2^x there is
 // below 1.2e-38, against 0 from ex2.approx.ftz).  Some of the pairs take
 // this path instead of MUFU ex2: the exponential step is bounded by the
@@ -566,6 +566,59 @@ __device__ __forceinline__ void ds32(const uint32_t (&pb)[16],
              r[2], r[3]);
     pd[2 * q] = pack_bf16(r[0], r[1]);
     pd[2 * q + 1] = pack_bf16(r[2], r[3]);
+  }
+}
+
+// The dQ kernel's forms of the two.  Its P enters no MMA, so it stays in fp32
+// and in place: rounded to bf16 pairs and widened again it took three of the
+// four ALU instructions per pair of columns in the two phases, which set the
+// step's pace (1650 clk against 840 of MMAs at d = 64, 1536 at d = 128).  Crop
+// training step 142.8 -> 138.1 us, clip 2271 -> 2235; with one rounding less
+// dQ's error against 64 bits falls from 2.9e-3 to 2.4e-3 (crop).  nl and nd are
+// the row's own -lse2 and -D.
+template <bool kMask>
+__device__ __forceinline__ void p32_row(uint32_t (&s)[32], float nl, int c0,
+                                        int lo, int hi, uint64_t c2x2) {
+  const uint64_t nl2 = f2(nl, nl);
+#pragma unroll
+  for (int q = 0; q < 8; ++q) {  // four columns at a time
+    float x[4];
+#pragma unroll
+    for (int u = 0; u < 4; u += 2)
+      f2_split(f2_fma(f2(__uint_as_float(s[4 * q + u]),
+                         __uint_as_float(s[4 * q + u + 1])),
+                      c2x2, nl2), x[u], x[u + 1]);
+    if (kMask) {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) {
+        const int col = c0 + 4 * q + u;
+        if (col < lo || col >= hi) x[u] = -INFINITY;
+      }
+    }
+    if (!kMask && poly_group(q)) {
+      exp2_poly(x[0], x[1]);
+      exp2_poly(x[2], x[3]);
+    } else {
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = ex2(x[u]);
+    }
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s[4 * q + u] = __float_as_uint(x[u]);
+  }
+}
+
+__device__ __forceinline__ void ds32_row(const uint32_t (&pf)[32],
+                                         const uint32_t (&dp)[32], float nd,
+                                         uint32_t (&pd)[16]) {
+  const uint64_t nd2 = f2(nd, nd);
+#pragma unroll
+  for (int q = 0; q < 16; ++q) {
+    float r0, r1;
+    f2_split(f2_mul(f2(__uint_as_float(pf[2 * q]), __uint_as_float(pf[2 * q + 1])),
+                    f2_add(f2(__uint_as_float(dp[2 * q]),
+                              __uint_as_float(dp[2 * q + 1])), nd2)),
+             r0, r1);
+    pd[q] = pack_bf16(r0, r1);
   }
 }
 
@@ -890,13 +943,7 @@ dq_kernel(const __grid_constant__ BwdParams p) {
     query_sees(p, row, vis_lo, vis_hi);
     const int64_t rl = (int64_t)bh_row(p, b, h) * p.padded + row;
     const float nl_row = p.lse2[rl];  // -log2 LSE (padded rows hold 0)
-    float4 nl_v[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) nl_v[q] = make_float4(nl_row, nl_row, nl_row, nl_row);
     const float nd_row = p.delta[rl];  // -D
-    float4 nd_v[8];
-#pragma unroll
-    for (int q = 0; q < 8; ++q) nd_v[q] = make_float4(nd_row, nd_row, nd_row, nd_row);
     const uint64_t c2x2 = f2(p.scale_log2, p.scale_log2);
     bool ok = true;
     int p_arr = 0, ds_arr = 0;  // hand-offs made to the MMA warp
@@ -909,8 +956,8 @@ dq_kernel(const __grid_constant__ BwdParams p) {
       const bool need_mask =
           __any_sync(0xffffffffu, lo > 0 || hi < 64 || !in_range);
       const int lo_m = in_range ? lo : 64, hi_m = in_range ? hi : 0;
-      uint32_t x0[32], x1[32], pb0[16], pb1[16], pk[16];
-      // phase 1 (overlaps the dP MMAs): P (bf16 pairs) in registers; S is
+      uint32_t x0[32], x1[32], d0[32], d1[32], pk[16];
+      // phase 1 (overlaps the dP MMAs): P in registers, in fp32; S is
       // then free for the next tile (released as soon as it has been read, the
       // next S and dP ran beside P and cost it more than they gained: crop
       // training step 141.7 -> 143.8 us)
@@ -918,11 +965,11 @@ dq_kernel(const __grid_constant__ BwdParams p) {
       tmem_ld32(row_t + cs + 32, x1);
       tmem_wait_ld();
       if (need_mask) {
-        p32<true>(x0, nl_v, 0, lo_m, hi_m, c2x2, pb0);
-        p32<true>(x1, nl_v, 32, lo_m, hi_m, c2x2, pb1);
+        p32_row<true>(x0, nl_row, 0, lo_m, hi_m, c2x2);
+        p32_row<true>(x1, nl_row, 32, lo_m, hi_m, c2x2);
       } else {
-        p32<false>(x0, nl_v, 0, lo_m, hi_m, c2x2, pb0);
-        p32<false>(x1, nl_v, 32, lo_m, hi_m, c2x2, pb1);
+        p32_row<false>(x0, nl_row, 0, lo_m, hi_m, c2x2);
+        p32_row<false>(x1, nl_row, 32, lo_m, hi_m, c2x2);
       }
       tc_fence_before();
       compute_arrive(kBarP);
@@ -932,12 +979,12 @@ dq_kernel(const __grid_constant__ BwdParams p) {
       if (!(ok = wait_bar_warp(&S->dp_ready[j & 1], (j >> 1) & 1, S))) break;
       tc_fence_after();
       const uint32_t cp = dq_dp_col(j) + 64 * hf;
-      tmem_ld32(row_t + cp, x0);
-      tmem_ld32(row_t + cp + 32, x1);
+      tmem_ld32(row_t + cp, d0);
+      tmem_ld32(row_t + cp + 32, d1);
       tmem_wait_ld();
-      ds32(pb0, x0, nd_v, pk);
+      ds32_row(x0, d0, nd_row, pk);
       tmem_st16(row_t + cp, pk);
-      ds32(pb1, x1, nd_v, pk);
+      ds32_row(x1, d1, nd_row, pk);
       tmem_st16(row_t + cp + 16, pk);
       tmem_wait_st();
       tc_fence_before();
