@@ -473,9 +473,6 @@ __device__ __forceinline__ uint64_t f2_mul(uint64_t a, uint64_t b) {
   asm("mul.rn.f32x2 %0, %1, %2;" : "=l"(r) : "l"(a), "l"(b));
   return r;
 }
-__device__ __forceinline__ float bf16_lo(uint32_t v) { return __uint_as_float(v << 16); }
-__device__ __forceinline__ float bf16_hi(uint32_t v) { return __uint_as_float(v & 0xffff0000u); }
-
 // 2^x of both halves of a packed pair on the FMA pipe: x = n + f with n the
 // nearest integer (x + 1.5 * 2^23 rounds it into the low mantissa bits) and
 // f in [-0.5, 0.5]; 2^f by a degree-3 polynomial (a relative-error minimax
@@ -507,7 +504,11 @@ __device__ __forceinline__ void exp2_poly(float& x0, float& x1) {
 __device__ __forceinline__ constexpr bool poly_group(int q) { return q == 7; }
 
 // P = 2^(s c2 - lse2) for 32 columns [c0, c0 + 32) of a half row, packed to
-// bf16 pairs; with kMask, columns outside [lo, hi) are masked (p = 0).  nl
+// bf16 pairs for the dV MMA and, in s, in fp32 for dS (dS from the bf16 pairs
+// had to widen them again, two of three ALU instructions per pair of columns,
+// added P's rounding error to dK: training clip step, with the dQ kernel's
+// form below, 2244 -> 2203 us, dK's error against 64 bits 2.9e-3 -> 2.4e-3 at
+// d = 64); with kMask, columns outside [lo, hi) are masked (p = 0).  nl
 // holds -lse2 for the 32 columns, in registers: the dK/dV kernel reads its
 // per-column values from shared memory ahead of use, because the SMEM x SMEM
 // MMAs that run meanwhile take all of the shared-memory bandwidth and each
@@ -516,9 +517,8 @@ __device__ __forceinline__ constexpr bool poly_group(int q) { return q == 7; }
 // compares and a select per element on every tile (measured: twice the time
 // of the unmasked form), while only tiles that cross a chunk edge need it.
 template <bool kMask>
-__device__ __forceinline__ void p32(const uint32_t (&s)[32],
-                                    const float4 (&nl)[8], int c0, int lo,
-                                    int hi, uint64_t c2x2,
+__device__ __forceinline__ void p32(uint32_t (&s)[32], const float4 (&nl)[8],
+                                    int c0, int lo, int hi, uint64_t c2x2,
                                     uint32_t (&pp)[16]) {
 #pragma unroll
   for (int q = 0; q < 8; ++q) {  // four columns at a time
@@ -538,29 +538,32 @@ __device__ __forceinline__ void p32(const uint32_t (&s)[32],
     if (!kMask && poly_group(q)) {
       exp2_poly(x[0], x[1]);
       exp2_poly(x[2], x[3]);
-      pp[2 * q] = pack_bf16(x[0], x[1]);
-      pp[2 * q + 1] = pack_bf16(x[2], x[3]);
     } else {
-      pp[2 * q] = pack_bf16(ex2(x[0]), ex2(x[1]));
-      pp[2 * q + 1] = pack_bf16(ex2(x[2]), ex2(x[3]));
+#pragma unroll
+      for (int u = 0; u < 4; ++u) x[u] = ex2(x[u]);
     }
+    pp[2 * q] = pack_bf16(x[0], x[1]);
+    pp[2 * q + 1] = pack_bf16(x[2], x[3]);
+#pragma unroll
+    for (int u = 0; u < 4; ++u) s[4 * q + u] = __float_as_uint(x[u]);
   }
 }
 
-// dS = P (dP - D) for 32 columns: P as 16 bf16 pairs, dP fp32, nd holds -D
-// for the 32 columns in registers.
-__device__ __forceinline__ void ds32(const uint32_t (&pb)[16],
+// dS = P (dP - D) for 32 columns: P and dP in fp32, nd holds -D for the 32
+// columns in registers.
+__device__ __forceinline__ void ds32(const uint32_t (&pf)[32],
                                      const uint32_t (&dp)[32],
                                      const float4 (&nd)[8], uint32_t (&pd)[16]) {
 #pragma unroll
   for (int q = 0; q < 8; ++q) {
     const float4 g = nd[q];
     float r[4];
-    f2_split(f2_mul(f2(bf16_lo(pb[2 * q]), bf16_hi(pb[2 * q])),
+    f2_split(f2_mul(f2(__uint_as_float(pf[4 * q]), __uint_as_float(pf[4 * q + 1])),
                     f2_add(f2(__uint_as_float(dp[4 * q]),
                               __uint_as_float(dp[4 * q + 1])), f2(g.x, g.y))),
              r[0], r[1]);
-    f2_split(f2_mul(f2(bf16_lo(pb[2 * q + 1]), bf16_hi(pb[2 * q + 1])),
+    f2_split(f2_mul(f2(__uint_as_float(pf[4 * q + 2]),
+                       __uint_as_float(pf[4 * q + 3])),
                     f2_add(f2(__uint_as_float(dp[4 * q + 2]),
                               __uint_as_float(dp[4 * q + 3])), f2(g.z, g.w))),
              r[2], r[3]);
@@ -768,7 +771,7 @@ dkdv_kernel(const __grid_constant__ BwdParams p) {
       tc_fence_after();
       const int lo = vis_lo - i0, hi = vis_hi - i0;
       const bool need_mask = __any_sync(0xffffffffu, lo > 0 || hi < 64);
-      uint32_t x0[32], x1[32], pb0[16], pb1[16], pk[16];
+      uint32_t x0[32], x1[32], dp[32], pk[16];
       // phase 1: P^T over the first half of S^T (for the dV MMA) and in
       // registers (for dS: the next tile's S^T may overwrite it in TMEM as
       // soon as dV has run)
@@ -779,15 +782,15 @@ dkdv_kernel(const __grid_constant__ BwdParams p) {
         lb[q] = reinterpret_cast<const float4*>(nl + 32)[q];
       tmem_wait_ld();
       if (need_mask) {
-        p32<true>(x0, la, 0, lo, hi, c2x2, pb0);
-        tmem_st16(row_t + cs, pb0);
-        p32<true>(x1, lb, 32, lo, hi, c2x2, pb1);
+        p32<true>(x0, la, 0, lo, hi, c2x2, pk);
+        tmem_st16(row_t + cs, pk);
+        p32<true>(x1, lb, 32, lo, hi, c2x2, pk);
       } else {
-        p32<false>(x0, la, 0, lo, hi, c2x2, pb0);
-        tmem_st16(row_t + cs, pb0);
-        p32<false>(x1, lb, 32, lo, hi, c2x2, pb1);
+        p32<false>(x0, la, 0, lo, hi, c2x2, pk);
+        tmem_st16(row_t + cs, pk);
+        p32<false>(x1, lb, 32, lo, hi, c2x2, pk);
       }
-      tmem_st16(row_t + cs + 16, pb1);
+      tmem_st16(row_t + cs + 16, pk);
       tmem_wait_st();
       tc_fence_before();
       compute_arrive(kBarP);
@@ -798,15 +801,16 @@ dkdv_kernel(const __grid_constant__ BwdParams p) {
       for (int q = 0; q < 8; ++q) la[q] = reinterpret_cast<const float4*>(nd)[q];
       if (!(ok = wait_bar_warp(&S->dp_ready[0], j & 1, S))) break;
       tc_fence_after();
-      tmem_ld32(row_t + cp, x0);
-      tmem_ld32(row_t + cp + 32, x1);
+      tmem_ld32(row_t + cp, dp);
 #pragma unroll
       for (int q = 0; q < 8; ++q)
         lb[q] = reinterpret_cast<const float4*>(nd + 32)[q];
       tmem_wait_ld();
-      ds32(pb0, x0, la, pk);
+      ds32(x0, dp, la, pk);
+      tmem_ld32(row_t + cp + 32, dp);
       tmem_st16(row_t + cp, pk);
-      ds32(pb1, x1, lb, pk);
+      tmem_wait_ld();
+      ds32(x1, dp, lb, pk);
       tmem_st16(row_t + cp + 16, pk);
       tmem_wait_st();
       tc_fence_before();
