@@ -1,8 +1,7 @@
 // FastVR's one-step restoration update (Eq. `eq:one_step`): after the DiT
 // predicts the velocity v from the low-quality latent z_LQ at t = tau, the
 // restored latent is z_hat = z_LQ - sigma_tau * v.  Elementwise and purely
-// bandwidth-bound: 16-byte loads of v (8 bf16) and of the matching z_LQ
-// elements, one fp32 FMA per element, a single rounding to the output type.
+// bandwidth-bound: 16-byte loads of z_LQ and of the matching elements of v, one fp32 FMA per element, a single rounding to the output type.
 #include <cuda_bf16.h>
 
 #include "fastvr_internal.h"
@@ -10,10 +9,17 @@
 namespace fastvr {
 namespace {
 
+// The elements of one thread's access: 16 bytes of z (8 bf16 or 4 fp32) and
+// the matching bf16 of v, so that a warp's accesses to each of the three
+// buffers are contiguous.  (8 fp32 in two 16-byte halves per thread, at a
+// stride of 32 bytes, touched every sector twice and wrote it in halves: 200 M
+// elements 324 us, now 299, 6.7 TB/s; 50 M 81.8 -> 75.6.)
 template <typename T>
-struct Vec8;  // 8 elements of T
+struct Vec;
 template <>
-struct Vec8<__nv_bfloat16> {
+struct Vec<__nv_bfloat16> {
+  static constexpr int kN = 8;
+  using V = uint4;
   uint4 u;
   __device__ float get(int i) const {
     const __nv_bfloat16* e = reinterpret_cast<const __nv_bfloat16*>(&u);
@@ -24,13 +30,17 @@ struct Vec8<__nv_bfloat16> {
   }
 };
 template <>
-struct Vec8<float> {
-  float4 a, b;
-  __device__ float get(int i) const {
-    return i < 4 ? (&a.x)[i] : (&b.x)[i - 4];
-  }
-  __device__ void set(int i, float x) { (i < 4 ? (&a.x)[i] : (&b.x)[i - 4]) = x; }
+struct Vec<float> {
+  static constexpr int kN = 4;
+  using V = uint2;
+  float4 a;
+  __device__ float get(int i) const { return (&a.x)[i]; }
+  __device__ void set(int i, float x) { (&a.x)[i] = x; }
 };
+template <typename V>
+__device__ __forceinline__ float bf16_at(const V& v, int i) {
+  return __bfloat162float(reinterpret_cast<const __nv_bfloat16*>(&v)[i]);
+}
 
 __device__ __forceinline__ float to_f(float x) { return x; }
 __device__ __forceinline__ float to_f(__nv_bfloat16 x) { return __bfloat162float(x); }
@@ -40,52 +50,60 @@ __device__ __forceinline__ void from_f(__nv_bfloat16& d, float x) {
 }
 
 // z and out may be the same buffer (in-place update): every element is read
-// and then written by the same thread.  Each thread keeps kUnroll groups of
-// loads in flight before it computes and stores, so that a few CTAs per SM
-// cover the HBM latency.
-constexpr int kUnroll = 4;
-
+// and then written by the same thread.  Each thread keeps a few groups of loads
+// in flight before it computes and stores, so that a few CTAs per SM cover the
+// HBM latency: 128 bytes at 4 bf16 or 8 fp32 groups, then, since a latent of a
+// few million elements gives a thread only two or three groups, two at a time.
 template <typename T>
-__device__ __forceinline__ void update8(const Vec8<T>& zv,
-                                        const Vec8<__nv_bfloat16>& vv,
-                                        float neg_sigma, Vec8<T>* dst) {
-  Vec8<T> o;
+__device__ __forceinline__ void update(const Vec<T>& zv,
+                                       const typename Vec<T>::V& vv,
+                                       float neg_sigma, Vec<T>* dst) {
+  Vec<T> o;
 #pragma unroll
-  for (int e = 0; e < 8; ++e) o.set(e, fmaf(neg_sigma, vv.get(e), zv.get(e)));
+  for (int e = 0; e < Vec<T>::kN; ++e)
+    o.set(e, fmaf(neg_sigma, bf16_at(vv, e), zv.get(e)));
   *dst = o;
+}
+
+// kU groups at a time, as long as that many are left; i moves on.
+template <int kU, typename T>
+__device__ __forceinline__ void run_groups(const Vec<T>* zg,
+                                           const typename Vec<T>::V* vg,
+                                           Vec<T>* og, int64_t& i,
+                                           int64_t groups, int64_t stride,
+                                           float neg_sigma) {
+  for (; i + (kU - 1) * stride < groups; i += kU * stride) {
+    Vec<T> zv[kU];
+    typename Vec<T>::V vv[kU];
+#pragma unroll
+    for (int u = 0; u < kU; ++u) {
+      zv[u] = zg[i + u * stride];
+      vv[u] = __ldcs(vg + i + u * stride);
+    }
+#pragma unroll
+    for (int u = 0; u < kU; ++u)
+      update(zv[u], vv[u], neg_sigma, og + i + u * stride);
+  }
 }
 
 template <typename T>
 __global__ void __launch_bounds__(256)
 one_step_kernel(const T* z, const __nv_bfloat16* __restrict__ v, T* out,
                 int64_t n, float neg_sigma) {
+  constexpr int kN = Vec<T>::kN;
   pdl_trigger();
   pdl_wait();  // z and v may come from the previous kernel on the stream
-  const int64_t n8 = n / 8;
+  const int64_t groups = n / kN;
   const int64_t stride = (int64_t)gridDim.x * blockDim.x;
   const int64_t tid = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-  const Vec8<T>* z8 = reinterpret_cast<const Vec8<T>*>(z);
-  const uint4* v8 = reinterpret_cast<const uint4*>(v);
-  Vec8<T>* o8 = reinterpret_cast<Vec8<T>*>(out);
+  const Vec<T>* zg = reinterpret_cast<const Vec<T>*>(z);
+  const typename Vec<T>::V* vg = reinterpret_cast<const typename Vec<T>::V*>(v);
+  Vec<T>* og = reinterpret_cast<Vec<T>*>(out);
   int64_t i = tid;
-  for (; i + (kUnroll - 1) * stride < n8; i += kUnroll * stride) {
-    Vec8<T> zv[kUnroll];
-    Vec8<__nv_bfloat16> vv[kUnroll];
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u) {
-      zv[u] = z8[i + u * stride];
-      vv[u].u = __ldcs(v8 + i + u * stride);
-    }
-#pragma unroll
-    for (int u = 0; u < kUnroll; ++u)
-      update8(zv[u], vv[u], neg_sigma, o8 + i + u * stride);
-  }
-  for (; i < n8; i += stride) {
-    Vec8<__nv_bfloat16> vv;
-    vv.u = __ldcs(v8 + i);
-    update8(z8[i], vv, neg_sigma, o8 + i);
-  }
-  for (int64_t i = n8 * 8 + tid; i < n; i += stride)  // fewer than 8 left
+  run_groups<32 / kN>(zg, vg, og, i, groups, stride, neg_sigma);
+  if (kN == 4) run_groups<2>(zg, vg, og, i, groups, stride, neg_sigma);
+  run_groups<1>(zg, vg, og, i, groups, stride, neg_sigma);
+  for (int64_t i = groups * kN + tid; i < n; i += stride)  // fewer than kN left
     from_f(out[i], fmaf(neg_sigma, __bfloat162float(v[i]), to_f(z[i])));
 }
 
@@ -99,7 +117,7 @@ cudaError_t launch_one_step(const void* z, const void* v, void* out, int64_t n,
   cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
   if (sms <= 0) sms = 152;
   int64_t blocks = (int64_t)sms * 8;
-  const int64_t need = (n / 8 + 255) / 256 + 1;
+  const int64_t need = (n / (dtype == 0 ? 8 : 4) + 255) / 256 + 1;
   if (blocks > need) blocks = need;
   const float neg_sigma = -sigma;
   if (dtype == 0)
