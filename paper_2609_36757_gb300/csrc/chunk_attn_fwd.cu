@@ -7,8 +7,8 @@
 // launch, invisible chunks are never loaded) and the only in-kernel mask is
 // the ragged end of a segment.
 //
-// One CTA owns two 128-row query tiles of one (batch, head) and streams the
-// visible keys in 128-key tiles:
+// One CTA owns two 128-row query tiles of one (batch, head), or one where a
+// launch has few, and streams the visible keys in 128-key tiles:
 //   warp 8      TMA producer of the Q tiles (once) and the K ring (3 deep);
 //   warp 10     TMA producer of the V ring (2 deep); all tiles are
 //               128-byte swizzled boxes of 64 columns.
@@ -131,10 +131,11 @@ struct TcParams {
   uint64_t wait_limit_ns;
   int32_t inject_stall;
   // Work split: units of two query tiles, (b, h, pair) with the pair index
-  // fastest, a head's last pair that holds one query tile only (long_pairs)
-  // after all others; the first units_full run whole, the tail_units after
-  // them are cut into `split` key-tile ranges, equal ones or, with cut > 0,
-  // [0, cut) and the rest, whose partial results go to the workspace.
+  // fastest, a head's last pair that holds one query tile only (pair
+  // long_pairs) after all others, or in its place (long_pairs = q_pairs); the
+  // first units_full run whole, the tail_units after them are cut into `split`
+  // key-tile ranges, equal ones or, with cut > 0, [0, cut) and the rest, whose
+  // partial results go to the workspace.
   int32_t q_pairs, long_pairs, units_full, tail_units, split, cut;
   int32_t unit_rows;  // query rows of a unit: two tiles, or one (few units)
   int32_t sms;  // SM count: CTA index / sms is a CTA's wave
@@ -202,7 +203,8 @@ __device__ __forceinline__ Work oneshot_work(const TcParams& p) {
   return w;
 }
 
-// Streaming: query pair and (b, h) of a unit; the short units come last.
+// Streaming: query pair and (b, h) of a unit; the short units come last, or,
+// with long_pairs = q_pairs, in their place.
 __device__ __forceinline__ void unit_coord(const TcParams& p, int unit,
                                            int& pair, int& bh) {
   const int n_long = p.long_pairs * p.heads * p.batch;
@@ -1123,6 +1125,12 @@ struct Split {
 // softmax and PV follow one another (480p, 25 to 199 key tiles: 0.72-0.78).
 constexpr double kOneTileCost = 0.75;
 
+// Launches whose units have at most this many key tiles run a head's unit of
+// one query tile after all others: it is the cheaper one to have left over
+// (480p, chunk of 25 tiles: 49.5 -> 43.1 us; no slower up to its 199 tiles).  Run there, away from its head's other units, it reads the
+// head's keys once more; at 720p's 450 tiles the launch is 0.7 % slower for it.
+constexpr int kShortsLastTiles = 256;
+
 // Whole waves of units run whole; the units of a last partial wave are cut
 // along the keys where that ends sooner.  Counted in key tiles of two query
 // tiles (about 1.1 us at d = 128): a CTA costs its tiles and kCtaCost (set-up,
@@ -1255,8 +1263,9 @@ cudaError_t launch_d(const AttnParams& a, cudaStream_t stream, int* launches) {
                                p.sms, split_parts(D));
   p.unit_rows = sp.unit_rows;
   p.q_pairs = units_of(a.q_tokens, sp.unit_rows);
-  p.long_pairs =
-      sp.unit_rows == kUnitRows ? long_pairs(a.q_tokens) : p.q_pairs;
+  p.long_pairs = sp.unit_rows == kUnitRows && tiles <= kShortsLastTiles
+                     ? long_pairs(a.q_tokens)
+                     : p.q_pairs;
   p.units_full = sp.units_full;
   p.tail_units = p.q_pairs * bh - sp.units_full;
   p.split = sp.split;

@@ -133,6 +133,10 @@ SPLITS = [
     WL.custom("whole-wave", batch=2, heads=76, head_dim=128,
               tokens_per_frame=70, frames_per_chunk=2, num_chunks=3,
               last_chunk_frames=1, seed=84),
+    # 195 units, 3 of them short: last over 129 key tiles, in place over 258
+    WL.custom("short-in-place", batch=1, heads=3, head_dim=64,
+              tokens_per_frame=16500, frames_per_chunk=1, num_chunks=2,
+              seed=85),
 ]
 
 
