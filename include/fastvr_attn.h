@@ -168,10 +168,10 @@ FASTVR_API fastvr_status_t fastvr_plan_visible(fastvr_plan_t plan, int32_t* num_
  * N; out bfloat16 [B, L, H, d]; lse nullable, float32 [B, H, L].  Frame f
  * belongs to chunk f / k; a ragged final chunk is simply shorter.  Each
  * block of 256 query rows (128 where the launch has few) reads only the keys
- * its rows can see (invisible chunks are never loaded); rows that straddle a chunk boundary are masked
- * element-wise.  No plan, no cache and no scratch memory are involved; a
- * bounded-wait timeout leaves out undefined and is reported by
- * fastvr_get_device_status.  The result
+ * its rows can see (invisible chunks are never loaded); rows that straddle a
+ * chunk boundary are masked element-wise.  No plan, no cache and no scratch
+ * memory are involved; a bounded-wait timeout leaves out undefined and is
+ * reported by fastvr_get_device_status.  The result
  * equals the streamed form (fastvr_kv_append + fastvr_chunk_attn_fwd, chunk
  * by chunk) up to rounding.
  * Errors: INVALID_ARG, UNSUPPORTED (head_dim, device not sm_103), CUDA. */

@@ -1127,8 +1127,9 @@ constexpr double kOneTileCost = 0.75;
 
 // Launches whose units have at most this many key tiles run a head's unit of
 // one query tile after all others: it is the cheaper one to have left over
-// (480p, chunk of 25 tiles: 49.5 -> 43.1 us; no slower up to its 199 tiles).  Run there, away from its head's other units, it reads the
-// head's keys once more; at 720p's 450 tiles the launch is 0.7 % slower for it.
+// (480p, chunk of 25 tiles: 49.5 -> 43.1 us; no slower up to its 199 tiles).
+// Run there, away from its head's other units, it reads the head's keys once
+// more; at 720p's 450 tiles the launch is 0.7 % slower for it.
 constexpr int kShortsLastTiles = 256;
 
 // Whole waves of units run whole; the units of a last partial wave are cut
@@ -1136,12 +1137,12 @@ constexpr int kShortsLastTiles = 256;
 // tiles (about 1.1 us at d = 128): a CTA costs its tiles and kCtaCost (set-up,
 // first loads, filling and draining the pipeline, epilogue: 10.8k clk against
 // 2240 per tile), the merge of the parts kMergeCost (its launch, here and on
-// the host, and its fixed time) and 1 / kPartsPerTile for each.  Equal parts may take more than one round on the SMs.  Where most of
-// the SMs have a unit already, two unequal parts: one for a CTA on each of
-// `rem` SMs, the others go round the rest, at most q on one SM, and the cut
-// lies where both end together.  (Equal parts in one round at most left 68 of
-// 152 SMs idle for a 480p frame, 84 units of 63 tiles:
-// 76.8 us, now 65.9 with the merge.)
+// the host, and its fixed time) and 1 / kPartsPerTile for each.  Equal parts
+// may take more than one round on the SMs.  Where most of the SMs have a unit
+// already, two unequal parts: one for a CTA on each of `rem` SMs, the others go
+// round the rest, at most q on one SM, and the cut lies where both end
+// together.  (Equal parts in one round at most left 68 of 152 SMs idle for a
+// 480p frame, 84 units of 63 tiles: 76.8 us, now 65.9 with the merge.)
 //
 // Where twice the units still fit the SMs, units of one query tile are the
 // other way to use more of them, and cost no merge (chunk of 600 queries x 2400

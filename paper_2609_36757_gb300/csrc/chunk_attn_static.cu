@@ -28,8 +28,8 @@
 
 namespace {
 
-// 24 MiB: room for 190 partial results at d = 128 (378 at d = 64); a GB300
-// launch uses at most one per SM (152).
+// 24 MiB: room for 190 partial results at d = 128 (378 at d = 64); a launch
+// leaves at most 190 (256 at d = 64), see split_parts.
 constexpr size_t kScratchBytes = fastvr::kStaticScratchBytes;
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];

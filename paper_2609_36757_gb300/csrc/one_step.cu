@@ -1,7 +1,8 @@
 // FastVR's one-step restoration update (Eq. `eq:one_step`): after the DiT
 // predicts the velocity v from the low-quality latent z_LQ at t = tau, the
 // restored latent is z_hat = z_LQ - sigma_tau * v.  Elementwise and purely
-// bandwidth-bound: 16-byte loads of z_LQ and of the matching elements of v, one fp32 FMA per element, a single rounding to the output type.
+// bandwidth-bound: 16-byte loads of z_LQ with the matching elements of v, one
+// fp32 FMA per element, a single rounding to the output type.
 #include <cuda_bf16.h>
 
 #include "fastvr_internal.h"
