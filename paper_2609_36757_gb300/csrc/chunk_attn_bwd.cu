@@ -38,6 +38,7 @@
 #include <mutex>
 
 #include "fastvr_internal.h"
+#include "handoff.h"
 #include "sm100_ptx.cuh"
 
 namespace fastvr {
@@ -48,9 +49,9 @@ using namespace sm100;
 constexpr int kT = 128;           // tile rows (TMEM lanes) and tile columns
 constexpr int kBox = 128 * 128;   // one TMA box: 128 rows x 64 bf16 (bytes)
 constexpr int kMaxStages = 3;     // deepest streamed ring
-constexpr int kStages1 = 2;       // ring 1 depth (ring 0: per kernel)
-constexpr int kDkdvS0 = 3;        // dK/dV ring 0 (Q)
-constexpr int kDqS0 = 3;          // dQ ring 0 (K): loads one step earlier
+constexpr int kStages1 = handoff::kBwdStages1;  // ring 1 depth
+constexpr int kDkdvS0 = handoff::kBwdStages0;   // dK/dV ring 0 (Q)
+constexpr int kDqS0 = handoff::kBwdStages0;  // dQ ring 0 (K): loads one step earlier
 constexpr int kThreads = 384;     // 8 compute warps, producer, MMA issuer,
                                   // relay, row-vector loader (dK/dV)
 constexpr int kProducerWarp = 8;
@@ -63,19 +64,10 @@ constexpr int kVecWarp = 11;
 // TMA loads have landed, the MMA warp syncs).  An mbarrier poll is a
 // shared-memory access that waits ~200 clk behind queued SMEM x SMEM MMAs;
 // a named barrier whose arrivals are in costs the MMA warp next to nothing.
-constexpr int kBarP = 1;
-constexpr int kBarDS = 2;
-constexpr int kBarRing0 = 3;  // + stage, up to kMaxStages
-constexpr int kBarRing1 = 6;  // + stage, up to kStages1
+// Which barrier is which, and their order: handoff.h.
 constexpr int kBarStaged = 8;  // the compute warps' output tiles are staged
-// The dQ kernel hands dS over through two barriers in turn (kBarDS, kBarDSOdd):
-// its next S and dP do not wait for dS, so a compute warp can be done with the
-// next dS while another has yet to arrive for this one, and on one barrier its
-// second arrival would stand in for the other's first.  It cannot be two ahead:
-// the S after that follows the MMA warp's wait for this dS.
-constexpr int kBarDSOdd = 9;
-constexpr int kComputeHandoff = 9 * 32;
-constexpr int kRelayHandoff = 2 * 32;
+constexpr int kComputeHandoff = handoff::kBwdComputeWarps * 32;
+constexpr int kRelayHandoff = handoff::kRelayWarps * 32;
 constexpr uint32_t kTmemCols = 512;
 constexpr uint64_t kWaitLimitNs = 4000000000ull;
 
@@ -230,28 +222,50 @@ __device__ __forceinline__ void relay_sync(int id) {
   asm volatile("bar.sync %0, %1;" ::"r"(id), "n"(kRelayHandoff) : "memory");
 }
 
+// The waits of a warp that makes the arrivals it owes after a failed wait
+// (handoff.h): deaf to the abort flag; past the limit, which only a stopped
+// tensor pipe reaches, the warp waits no more.
+struct OwedWaits {
+  bool pipe_runs = true;
+  __device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity) {
+    const uint64_t t0 = global_timer_ns();
+    while (pipe_runs) {
+      const bool late = global_timer_ns() - t0 > kWaitLimitNs;
+      if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return;
+      pipe_runs = !__any_sync(0xffffffffu, late);
+    }
+  }
+};
+
+// A commit of the MMA warp; with nothing issued, an arrival.
+template <bool kIssue>
+__device__ __forceinline__ void commit_step(uint64_t* bar) {
+  if (kIssue)
+    mma_commit_warp(bar);
+  else if ((threadIdx.x & 31) == 0)
+    mbar_arrive(bar);
+}
+
 // The relay warp observes each step's two streamed tiles (ring 0, then
 // ring 1, the order in which the MMA warp needs them) and hands each stage
 // over through its named barrier.  A stage's barrier cannot be arrived at
 // twice before the MMA warp has synced on it: the producer refills a stage
-// only after the MMAs that read it.  Named barriers have no time limit, so
-// after a failed wait the relay still makes the remaining arrivals (the
-// MMA warp then computes on undefined data; the failure is recorded).
-template <int kS0>
+// only after the MMAs that read it.
 __device__ void bwd_relay(BwdShared* S, int n) {
-  int a0 = 0, a1 = 0;
-  bool ok = true;
-  for (int j = 0; ok && j < n; ++j) {
-    if (!(ok = wait_bar_warp(&S->full[0][j % kS0], (j / kS0) & 1, S))) break;
-    relay_arrive(kBarRing0 + j % kS0);
-    ++a0;
-    if (!(ok = wait_bar_warp(&S->full[1][j % kStages1], (j / kStages1) & 1, S)))
-      break;
-    relay_arrive(kBarRing1 + j % kStages1);
-    ++a1;
-  }
-  for (; a0 < n; ++a0) relay_arrive(kBarRing0 + a0 % kS0);
-  for (; a1 < n; ++a1) relay_arrive(kBarRing1 + a1 % kStages1);
+  struct Ops {
+    BwdShared* S;
+    OwedWaits owed;
+    __device__ __forceinline__ bool wait(int ring, int j) {
+      const int depth = ring ? kStages1 : handoff::kBwdStages0;
+      return wait_bar_warp(&S->full[ring][j % depth], (j / depth) & 1, S);
+    }
+    __device__ __forceinline__ void wait_slot(int ring, int j) {
+      const int depth = ring ? kStages1 : handoff::kBwdStages0;
+      owed.wait(&S->empty[ring][j % depth], ((j / depth) & 1) ^ 1);
+    }
+    __device__ __forceinline__ void arrive(int id) { relay_arrive(id); }
+  } ops{S, {}};
+  handoff::bwd_relay_steps(n, ops);
 }
 
 __device__ __forceinline__ void drain_wait(uint64_t* bar, uint32_t parity) {
@@ -625,6 +639,63 @@ __device__ __forceinline__ void ds32_row(const uint32_t (&pf)[32],
   }
 }
 
+// What a compute warp owes after a failed wait (handoff::bwd_compute_rest); the
+// dQ kernel's dP has two buffers.
+template <bool kTwoDp>
+struct OwedCompute {
+  BwdShared* S;
+  OwedWaits owed;
+  __device__ __forceinline__ void wait_s(int j) {
+    owed.wait(&S->s_ready, j & 1);
+  }
+  __device__ __forceinline__ void wait_dp(int j) {
+    owed.wait(&S->dp_ready[kTwoDp ? j & 1 : 0], (kTwoDp ? j >> 1 : j) & 1);
+  }
+  __device__ __forceinline__ void arrive(int id) { compute_arrive(id); }
+};
+
+// What the dK/dV kernel's MMA warp does between its hand-offs
+// (handoff::dkdv_mma_steps); with kIssue false, after a wait that failed before
+// the first MMA, the commits alone.
+//
+// The next tile's S^T is issued right after this tile's dV (it overwrites P^T, which dV has read: the pipe runs in issue order
+// and the compute warps keep P^T in registers), and the next dP^T right
+// after dK (over dS^T), so the compute warps start the next tile's P
+// as soon as they finish this tile's dS.  Q (ring 0) and dO (ring 1) run at
+// their own depths.
+template <int D, bool kIssue>
+struct DkdvMmaOps {
+  using L = DkdvLayout<D>;
+  BwdShared* S;
+  uint32_t sbase, tmem;
+  __device__ __forceinline__ void relay_sync(int id) { fastvr::relay_sync(id); }
+  __device__ __forceinline__ void compute_sync(int id) {
+    fastvr::compute_sync(id);
+  }
+  __device__ __forceinline__ void s(int j) {  // S^T_j = K Q_j^T
+    tc_fence_after();
+    if (kIssue) mma_nt<D, L>(sbase, tmem, 0, 0, j % kDkdvS0, 0);
+    commit_step<kIssue>(&S->s_ready);
+  }
+  __device__ __forceinline__ void dp(int j) {  // dP^T_j = V dO_j^T
+    tc_fence_after();
+    if (kIssue) mma_nt<D, L>(sbase, tmem, 128, 1, j % kStages1, 1);
+    commit_step<kIssue>(&S->dp_ready[0]);
+  }
+  __device__ __forceinline__ void dv(int j) {
+    tc_fence_after();
+    if (kIssue)
+      mma_tn<D>(sbase, tmem, 256, 0, L::ring(j % kStages1, 1, 0), j > 0);
+    commit_step<kIssue>(&S->empty[1][j % kStages1]);  // dO_j's last reader
+  }
+  __device__ __forceinline__ void out(int j) {  // dK
+    tc_fence_after();
+    if (kIssue)
+      mma_tn<D>(sbase, tmem, 384, 128, L::ring(j % kDkdvS0, 0, 0), j > 0);
+    commit_step<kIssue>(&S->empty[0][j % kDkdvS0]);  // Q_j's last reader
+  }
+};
+
 // ------------------------------------------------------------------ dK, dV
 // TMEM: [0,128) S^T then P^T (bf16, first 64 columns), [128,256) dP^T then
 // dS^T, [256,256+d) dV, [384,384+d) dK.  Resident: K (fixed 0), V (fixed 1).
@@ -670,7 +741,7 @@ dkdv_kernel(const __grid_constant__ BwdParams p) {
                       q0, n, h, b);
     __syncwarp();
   } else if (warp == kRelayWarp) {
-    bwd_relay<kDkdvS0>(S, n);
+    bwd_relay(S, n);
   } else if (warp == kVecWarp) {
     // Row vectors: step j's 128 -log2 LSE and -D values into slot j % 2,
     // once the compute warps have released the slot (after dS of step j-2).
@@ -693,51 +764,17 @@ dkdv_kernel(const __grid_constant__ BwdParams p) {
     __syncwarp();
   } else if (warp == kMmaWarp) {
     const uint32_t sbase = smem_addr(smem);
-    // The next tile's S^T is issued right after this tile's dV (it
-    // overwrites P^T, which dV has read: the pipe runs in issue order and
-    // the compute warps keep P^T in registers), and the next dP^T right
-    // after dK (over dS^T), so the compute warps start the next tile's P
-    // as soon as they finish this tile's dS.
     // Test hook: o_full receives no arrival before the end, so this wait
     // runs out and exercises the abort path.
-    bool ok = (!p.inject_stall || wait_bar_warp(&S->o_full, 0, S)) &&
-              wait_bar_warp(&S->fixed_full, 0, S);
-    if (ok) {
-      relay_sync(kBarRing0);
-      tc_fence_after();
-      mma_nt<D, L>(sbase, tmem, 0, 0, 0, 0);    // S^T_0 = K Q_0^T
-      mma_commit_warp(&S->s_ready);
-      relay_sync(kBarRing1);
-      tc_fence_after();
-      mma_nt<D, L>(sbase, tmem, 128, 1, 0, 1);  // dP^T_0 = V dO_0^T
-      mma_commit_warp(&S->dp_ready[0]);
+    if ((!p.inject_stall || wait_bar_warp(&S->o_full, 0, S)) &&
+        wait_bar_warp(&S->fixed_full, 0, S)) {
+      DkdvMmaOps<D, true> ops{S, sbase, tmem};
+      handoff::dkdv_mma_steps(n, ops);
+      mma_commit_warp(&S->o_full);
+    } else {
+      DkdvMmaOps<D, false> ops{S, sbase, tmem};
+      handoff::dkdv_mma_steps(n, ops);
     }
-    for (int j = 0; ok && j < n; ++j) {
-      // Q (ring 0) and dO (ring 1) run at their own depths
-      const int q_st = j % kDkdvS0, q_stn = (j + 1) % kDkdvS0;
-      const int o_st = j % kStages1, o_stn = (j + 1) % kStages1;
-      compute_sync(kBarP);
-      tc_fence_after();
-      mma_tn<D>(sbase, tmem, 256, 0, L::ring(o_st, 1, 0), j > 0);    // dV
-      mma_commit_warp(&S->empty[1][o_st]);  // dO_j read for the last time
-      if (j + 1 < n) {
-        relay_sync(kBarRing0 + q_stn);
-        tc_fence_after();
-        mma_nt<D, L>(sbase, tmem, 0, 0, q_stn, 0);  // S^T_{j+1}
-        mma_commit_warp(&S->s_ready);
-      }
-      compute_sync(kBarDS);
-      tc_fence_after();
-      mma_tn<D>(sbase, tmem, 384, 128, L::ring(q_st, 0, 0), j > 0);  // dK
-      mma_commit_warp(&S->empty[0][q_st]);  // Q_j read for the last time
-      if (j + 1 < n) {
-        relay_sync(kBarRing1 + o_stn);
-        tc_fence_after();
-        mma_nt<D, L>(sbase, tmem, 128, 1, o_stn, 1);  // dP^T_{j+1}
-        mma_commit_warp(&S->dp_ready[0]);
-      }
-    }
-    if (ok) mma_commit_warp(&S->o_full);
     mma_commit_warp(&S->drain);
     if (lane == 0) drain_wait(&S->drain, 0);
     __syncwarp();
@@ -793,7 +830,7 @@ dkdv_kernel(const __grid_constant__ BwdParams p) {
       tmem_st16(row_t + cs + 16, pk);
       tmem_wait_st();
       tc_fence_before();
-      compute_arrive(kBarP);
+      compute_arrive(handoff::kBwdP);
       ++p_arr;
       // phase 2 (overlaps the dV and next S^T MMAs): dS^T over the first
       // half of dP^T; the D values are read ahead like the LSE values
@@ -814,17 +851,15 @@ dkdv_kernel(const __grid_constant__ BwdParams p) {
       tmem_st16(row_t + cp + 16, pk);
       tmem_wait_st();
       tc_fence_before();
-      compute_arrive(kBarDS);
+      compute_arrive(handoff::bwd_ds(j, false));
       ++ds_arr;
       // the row-vector slot is read for the last time
       __syncwarp();
       if (lane == 0) mbar_arrive(&S->vec_empty[sl]);
     }
-    // After a failed wait the remaining hand-offs are still made (with
-    // undefined contents), so that the MMA warp never waits for an arrival
-    // that does not come.
-    for (; p_arr < n; ++p_arr) compute_arrive(kBarP);
-    for (; ds_arr < n; ++ds_arr) compute_arrive(kBarDS);
+    if (!ok)
+      handoff::bwd_compute_rest(n, false, p_arr, ds_arr,
+                                OwedCompute<false>{S, {}});
     // dV and dK are staged in the first two Q stages (free once o_full has
     // completed: every MMA has read its operands) and leave as TMA stores;
     // rows past the sequence fall outside the map and are not written.
@@ -853,6 +888,42 @@ dkdv_kernel(const __grid_constant__ BwdParams p) {
 // columns) for even and odd steps, [256,256+d) dQ.  Resident: Q (fixed 0),
 // dO (fixed 1).  Streamed: K (ring 0), V (ring 1).
 __device__ __forceinline__ int dq_dp_col(int j) { return (j & 1) ? 384 : 128; }
+
+// What its MMA warp does between its hand-offs (handoff::dq_mma_steps).
+//
+// S and dP of the next tile are issued as soon as P of this one is in
+// registers, so they overlap the dS computation; dP alternates between
+// two buffers, so it need not wait for this tile's dQ to read dS (dP_{j+1}
+// goes to the buffer that dQ_{j-1}, issued before, read).  K (ring 0) and V
+// (ring 1) run at their own depths.
+template <int D, bool kIssue>
+struct DqMmaOps {
+  using L = BwdLayout<D, kDqS0>;
+  BwdShared* S;
+  uint32_t sbase, tmem;
+  __device__ __forceinline__ void relay_sync(int id) { fastvr::relay_sync(id); }
+  __device__ __forceinline__ void compute_sync(int id) {
+    fastvr::compute_sync(id);
+  }
+  __device__ __forceinline__ void s(int j) {  // S_j = Q K_j^T
+    tc_fence_after();
+    if (kIssue) mma_nt<D, L>(sbase, tmem, 0, 0, j % kDqS0, 0);
+    commit_step<kIssue>(&S->s_ready);
+  }
+  __device__ __forceinline__ void dp(int j) {  // dP_j = dO V_j^T
+    tc_fence_after();
+    if (kIssue) mma_nt<D, L>(sbase, tmem, dq_dp_col(j), 1, j % kStages1, 1);
+    commit_step<kIssue>(&S->dp_ready[j & 1]);
+    commit_step<kIssue>(&S->empty[1][j % kStages1]);  // V_j's last reader
+  }
+  __device__ __forceinline__ void out(int j) {  // dQ
+    tc_fence_after();
+    if (kIssue)
+      mma_tn<D>(sbase, tmem, 256, dq_dp_col(j), L::ring(j % kDqS0, 0, 0), j > 0);
+    commit_step<kIssue>(&S->empty[0][j % kDqS0]);  // K_j's last reader
+  }
+};
+
 template <int D>
 __global__ void __launch_bounds__(kThreads, 1)
 dq_kernel(const __grid_constant__ BwdParams p) {
@@ -880,56 +951,23 @@ dq_kernel(const __grid_constant__ BwdParams p) {
                       kv0, n, h, b);
     __syncwarp();
   } else if (warp == kRelayWarp) {
-    bwd_relay<kDqS0>(S, n);
+    bwd_relay(S, n);
   } else if (warp == kVecWarp) {
     // no row-vector warp here: each compute thread reads its own row's two
     // values once
   } else if (warp == kMmaWarp) {
     const uint32_t sbase = smem_addr(smem);
-    // S and dP of the next tile are issued as soon as P of this one is in
-    // registers, so they overlap the dS computation; dP alternates between
-    // two buffers, so it need not wait for this tile's dQ to read dS.
     // Test hook: o_full receives no arrival before the end, so this wait
     // runs out and exercises the abort path.
-    bool ok = (!p.inject_stall || wait_bar_warp(&S->o_full, 0, S)) &&
-              wait_bar_warp(&S->fixed_full, 0, S);
-    if (ok) {
-      relay_sync(kBarRing0);
-      tc_fence_after();
-      mma_nt<D, L>(sbase, tmem, 0, 0, 0, 0);    // S_0 = Q K_0^T
-      mma_commit_warp(&S->s_ready);
-      relay_sync(kBarRing1);
-      tc_fence_after();
-      mma_nt<D, L>(sbase, tmem, dq_dp_col(0), 1, 0, 1);  // dP_0 = dO V_0^T
-      mma_commit_warp(&S->dp_ready[0]);
-      mma_commit_warp(&S->empty[1][0]);  // V_0 read for the last time
+    if ((!p.inject_stall || wait_bar_warp(&S->o_full, 0, S)) &&
+        wait_bar_warp(&S->fixed_full, 0, S)) {
+      DqMmaOps<D, true> ops{S, sbase, tmem};
+      handoff::dq_mma_steps(n, ops);
+      mma_commit_warp(&S->o_full);
+    } else {
+      DqMmaOps<D, false> ops{S, sbase, tmem};
+      handoff::dq_mma_steps(n, ops);
     }
-    for (int j = 0; ok && j < n; ++j) {
-      // K (ring 0) and V (ring 1) run at their own depths
-      const int k_st = j % kDqS0, k_stn = (j + 1) % kDqS0;
-      const int v_stn = (j + 1) % kStages1;
-      compute_sync(kBarP);
-      if (j + 1 < n) {
-        relay_sync(kBarRing0 + k_stn);
-        tc_fence_after();
-        mma_nt<D, L>(sbase, tmem, 0, 0, k_stn, 0);  // S_{j+1}
-        mma_commit_warp(&S->s_ready);
-        // dP_{j+1} goes to the buffer that dQ_{j-1} (issued before) read
-        relay_sync(kBarRing1 + v_stn);
-        tc_fence_after();
-        mma_nt<D, L>(sbase, tmem, dq_dp_col(j + 1), 1, v_stn, 1);
-        mma_commit_warp(&S->dp_ready[(j + 1) & 1]);
-        mma_commit_warp(&S->empty[1][v_stn]);  // V_{j+1} read for the last time
-      }
-      if (j & 1)
-        compute_sync(kBarDSOdd);
-      else
-        compute_sync(kBarDS);
-      tc_fence_after();
-      mma_tn<D>(sbase, tmem, 256, dq_dp_col(j), L::ring(k_st, 0, 0), j > 0);  // dQ
-      mma_commit_warp(&S->empty[0][k_st]);  // K_j read for the last time
-    }
-    if (ok) mma_commit_warp(&S->o_full);
     mma_commit_warp(&S->drain);
     if (lane == 0) drain_wait(&S->drain, 0);
     __syncwarp();
@@ -976,7 +1014,7 @@ dq_kernel(const __grid_constant__ BwdParams p) {
         p32_row<false>(x1, nl_row, 32, lo_m, hi_m, c2x2);
       }
       tc_fence_before();
-      compute_arrive(kBarP);
+      compute_arrive(handoff::kBwdP);
       ++p_arr;
       // phase 2 (overlaps the next tile's S and dP MMAs): dS over this
       // step's dP buffer
@@ -992,18 +1030,12 @@ dq_kernel(const __grid_constant__ BwdParams p) {
       tmem_st16(row_t + cp + 16, pk);
       tmem_wait_st();
       tc_fence_before();
-      if (j & 1)
-        compute_arrive(kBarDSOdd);
-      else
-        compute_arrive(kBarDS);
+      compute_arrive(handoff::bwd_ds(j, true));
       ++ds_arr;
     }
-    // After a failed wait the remaining hand-offs are still made (with
-    // undefined contents), so that the MMA warp never waits for an arrival
-    // that does not come.
-    for (; p_arr < n; ++p_arr) compute_arrive(kBarP);
-    for (; ds_arr < n; ++ds_arr)
-      compute_arrive(ds_arr & 1 ? kBarDSOdd : kBarDS);
+    if (!ok)
+      handoff::bwd_compute_rest(n, true, p_arr, ds_arr,
+                                OwedCompute<true>{S, {}});
     // dQ is staged in the first K stage (free once o_full has completed)
     // and leaves as TMA stores; rows past the sequence are not written.
     uint8_t* const tiles[1] = {smem + L::ring(0, 0, 0)};

@@ -28,7 +28,8 @@
 // which gives its softmax three MMA steps to store P_t.  The MMA warp never
 // polls a shared-memory barrier: every hand-off to it (S read, P_t stored,
 // K/V stage landed) is a named barrier, whose arrivals are made on every
-// path (also after a failed wait), since a named barrier has no time limit.
+// path (also after a failed wait: handoff.h), since a named barrier has no time
+// limit.
 //
 // Online softmax in the exp2 domain: each row keeps a reference m (a lower
 // bound of its running max) and exponentiates against it; m moves, and O is
@@ -54,6 +55,7 @@
 #include <algorithm>
 
 #include "fastvr_internal.h"
+#include "handoff.h"
 #include "sm100_ptx.cuh"
 
 namespace fastvr {
@@ -64,8 +66,8 @@ using namespace sm100;
 constexpr int kBM = 128;        // query rows per tile (one TMEM lane each)
 constexpr int kBN = 128;        // keys per tile
 constexpr int kQTiles = 2;      // query tiles per CTA
-constexpr int kKStages = 3;     // depth of the K ring
-constexpr int kVStages = 2;     // depth of the V ring
+constexpr int kKStages = handoff::kFwdKStages;  // depth of the K ring
+constexpr int kVStages = handoff::kFwdVStages;  // depth of the V ring
 constexpr int kThreads = 384;   // 8 softmax warps, K and V producers, MMA,
                                 // relay
 constexpr int kBox = 128 * 128; // one TMA box: 128 rows x 64 bf16 (bytes)
@@ -96,22 +98,13 @@ static_assert(Tmem<128>::o(1) + 128 == kTmemCols &&
 constexpr float kRescaleThreshold = 8.0f;      // log2 units
 constexpr int kMinTilesPerPart = 4;             // key tiles per split part
 constexpr uint64_t kDefaultWaitLimitNs = 4000000000ull;  // 4 s per wait
-// Named (hardware) barriers of the softmax -> MMA hand-offs: S read (free
-// for the next QK^T) and P_t stored.  The four softmax warps of a tile
-// arrive, the MMA warp syncs: kHandoff threads per generation.
-constexpr int kBarSFree = 1;
-constexpr int kBarPFull0 = 2;  // + t
-constexpr int kHandoff = 5 * 32;
-// Named barriers of the relay -> MMA hand-offs, one per ring stage: K (or V)
-// stage s has landed.  The relay warp arrives, the MMA warp syncs.
-constexpr int kBarKFull0 = 4;  // + stage (kKStages of them)
-constexpr int kBarVFull0 = 7;  // + stage (kVStages of them)
-constexpr int kRelay = 2 * 32;
+// Threads of a generation of the hand-offs' named barriers (which of them are
+// which, and their order: handoff.h).
+constexpr int kHandoff = handoff::kFwdSoftmaxWarps * 32;
+constexpr int kRelay = handoff::kRelayWarps * 32;
 // Named barrier of a query tile's four softmax warps: their rows of O are
 // staged for the tile's TMA store.
 constexpr int kBarOStaged0 = 9;  // + t
-// "S read" of query tile 1 where each tile has an S of its own (d = 64).
-constexpr int kBarSFree1 = 11;
 
 struct TcParams {
   CUtensorMap q_map;                  // {d, Lq, H, B}
@@ -403,13 +396,37 @@ __device__ __forceinline__ bool wait_bar_warp(uint64_t* bar, uint32_t parity,
   }
 }
 
+// The waits of a warp that makes the arrivals it owes after a failed wait
+// (handoff.h): deaf to the abort flag; past the limit, which only a stopped
+// tensor pipe reaches, the warp waits no more.
+struct OwedWaits {
+  bool pipe_runs = true;
+  __device__ __forceinline__ void wait(uint64_t* bar, uint32_t parity) {
+    const uint64_t t0 = global_timer_ns();
+    while (pipe_runs) {
+      const bool late = global_timer_ns() - t0 > kDefaultWaitLimitNs;
+      if (__all_sync(0xffffffffu, mbar_try_wait(bar, parity))) return;
+      pipe_runs = !__any_sync(0xffffffffu, late);
+    }
+  }
+};
+
+// A commit of the MMA warp; with nothing issued, an arrival.
+template <bool kIssue>
+__device__ __forceinline__ void commit_step(uint64_t* bar) {
+  if (kIssue)
+    mma_commit_warp(bar);
+  else if ((threadIdx.x & 31) == 0)
+    mbar_arrive(bar);
+}
+
 // Hand-offs from the softmax warps to the MMA warp go through named
 // barriers, which live in hardware rather than in shared memory: an mbarrier
 // poll is a shared-memory access, and while SMEM x SMEM MMAs are queued every
 // such access waits behind their operand reads (~200 clk), which the issuer
 // cannot afford several times per key tile.  A named barrier has no time
-// limit, so the softmax warps make exactly the arrivals the MMA warp will
-// wait for on every path, also after a failed wait (see softmax_role).
+// limit: after a failed wait a role still makes the arrivals that it owes, in
+// step with the MMA warp (handoff.h says how).
 __device__ __forceinline__ void named_arrive(int id) {
   asm volatile("bar.arrive %0, %1;" ::"r"(id), "n"(kHandoff) : "memory");
 }
@@ -432,133 +449,109 @@ __device__ __forceinline__ void relay_sync(int id) {
 // barrier of its ring stage, so the MMA warp itself never polls a
 // shared-memory barrier.  A stage's barrier cannot be arrived at twice
 // before the MMA warp has synced on it: the producer refills the stage only
-// after the MMAs that read it.  After a failed wait the remaining arrivals
-// are still made (the MMA warp then computes on undefined data, and the
-// failure is recorded), so the MMA warp never waits for one that does not
-// come.
+// after the MMAs that read it.
 __device__ void relay_role(const TcParams& p, Shared* S, int n) {
-  int k_arr = 0, v_arr = 0;
-  bool ok = true;
-  for (int j = 0; ok && j <= n; ++j) {
-    if (j < n) {
-      if (!(ok = wait_bar_warp(&S->k_full[j % kKStages], (j / kKStages) & 1,
-                               S, p.status)))
-        break;
-      relay_arrive(kBarKFull0 + j % kKStages);
-      ++k_arr;
+  struct Ops {
+    Shared* S;
+    int* status;
+    OwedWaits owed;
+    __device__ __forceinline__ bool wait_k(int j) {
+      return wait_bar_warp(&S->k_full[j % kKStages], (j / kKStages) & 1, S,
+                           status);
     }
-    const int jp = j - 1;
-    if (jp >= 0) {
-      if (!(ok = wait_bar_warp(&S->v_full[jp % kVStages],
-                               (jp / kVStages) & 1, S, p.status)))
-        break;
-      relay_arrive(kBarVFull0 + jp % kVStages);
-      ++v_arr;
+    __device__ __forceinline__ bool wait_v(int j) {
+      return wait_bar_warp(&S->v_full[j % kVStages], (j / kVStages) & 1, S,
+                           status);
     }
-  }
-  for (; k_arr < n; ++k_arr) relay_arrive(kBarKFull0 + k_arr % kKStages);
-  for (; v_arr < n; ++v_arr) relay_arrive(kBarVFull0 + v_arr % kVStages);
+    __device__ __forceinline__ void wait_k_slot(int j) {
+      owed.wait(&S->k_empty[j % kKStages], ((j / kKStages) & 1) ^ 1);
+    }
+    __device__ __forceinline__ void wait_v_slot(int j) {
+      owed.wait(&S->v_empty[j % kVStages], ((j / kVStages) & 1) ^ 1);
+    }
+    __device__ __forceinline__ void arrive(int id) { relay_arrive(id); }
+  } ops{S, p.status, {}};
+  handoff::fwd_relay_steps(n, ops);
 }
 
+// What the MMA warp does between its hand-offs (handoff::fwd_mma_steps); with
+// kIssue false, after a wait that failed before the first MMA, the commits
+// alone.
+//
+// One warp issues every MMA (an elected lane, the warp kept converged) and
+// a tcgen05.mma takes it ~54 clk to issue against 64 clk of tensor work
+// (M128 N128 K16), so the issue loop carries no descriptor arithmetic: the
+// descriptor words are formed once and each MMA only adds a constant
+// offset (16-byte units) to the low word.
+template <int D, bool kIssue>
+struct MmaOps {
+  using L = Layout<D>;
+  using T = Tmem<D>;
+  static constexpr uint32_t kIdescQK = idesc_bf16_f32(kBM, kBN, 0);
+  static constexpr uint32_t kIdescPV = idesc_bf16_f32(kBM, D, 1);
+  static constexpr uint32_t kStage16 = (uint32_t)(L::kNB * kBox) >> 4;
+  Shared* S;
+  uint32_t tmem, hi, q_lo, k_lo, v_lo;
+
+  __device__ __forceinline__ void relay_sync(int id) {
+    fastvr::relay_sync(id);
+  }
+  __device__ __forceinline__ void softmax_sync(int id) { named_sync(id); }
+  // S_t = Q_t K^T: both operands K-major, 128-byte
+  // swizzle; a K step of 16 elements is 32 bytes inside a 64-column box.
+  __device__ __forceinline__ void qk(int t, int st, bool last_use) {
+    tc_fence_after();
+    const uint32_t a0 = q_lo + (uint32_t)(L::q(t, 0) >> 4);
+    const uint32_t b0 = k_lo + (uint32_t)st * kStage16;
+#pragma unroll
+    for (int ks = 0; kIssue && ks < D / 16; ++ks) {
+      const uint32_t off = (uint32_t)((ks / 4) * kBox + (ks % 4) * 32) >> 4;
+      mma_ss_warp(tmem + T::s(t), a0 + off, b0 + off, hi, kIdescQK, ks > 0);
+    }
+    commit_step<kIssue>(&S->s_full[t]);
+    if (last_use) commit_step<kIssue>(&S->k_empty[st]);
+  }
+  // O_t += P_t V: P_t from its TMEM columns (8 per 16 keys), V MN-major (d
+  // contiguous): 16 keys are two 8-row groups (2048 bytes), the two 64-column
+  // halves of d are one box apart.
+  __device__ __forceinline__ void pv(int t, int st, bool acc, bool last_use) {
+    tc_fence_after();
+    const uint32_t b0 = v_lo + (uint32_t)st * kStage16;
+#pragma unroll
+    for (int kk = 0; kIssue && kk < kBN / 16; ++kk)
+      mma_ts_warp(tmem + T::o(t), tmem + T::p(t) + kk * 8,
+                  b0 + (uint32_t)(kk * 2048 >> 4), hi, kIdescPV,
+                  (acc | kk) != 0);
+    commit_step<kIssue>(&S->p_free[t]);
+    if (last_use) commit_step<kIssue>(&S->v_empty[st]);
+  }
+};
+
+// Issue order per key tile j: QK_0(j), PV_0(j-1), QK_1(j), PV_1(j-1).  A
+// tile's PV runs one key tile behind its QK^T, so the softmax of S_t(j)
+// has the MMAs of three other steps (about 2000 clk) to produce P_t(j)
+// before the pipe needs it, while S, which only has to survive until the
+// softmax has loaded it, alternates between the tiles.
 template <int D>
 __device__ void mma_issuer(const TcParams& p, uint8_t* smem, Shared* S,
                            uint32_t tmem, const Work& w) {
   using L = Layout<D>;
-  using T = Tmem<D>;
-  constexpr uint32_t kIdescQK = idesc_bf16_f32(kBM, kBN, 0);
-  constexpr uint32_t kIdescPV = idesc_bf16_f32(kBM, D, 1);
   const uint32_t sbase = smem_addr(smem);
-  const int n = w.n;
-  const bool two = w.nqt == 2;
-
-  // One warp issues every MMA (an elected lane, the warp kept converged) and
-  // a tcgen05.mma takes it ~54 clk to issue against 64 clk of tensor work
-  // (M128 N128 K16), so the issue loop carries no descriptor arithmetic: the
-  // descriptor words are formed once here and each MMA only adds a constant
-  // offset (16-byte units) to the low word.
-  const uint32_t hi = desc_hi_sw128(1024);
-  const uint32_t q_lo = desc_lo(sbase + L::q(0, 0), 16);
-  const uint32_t k_lo = desc_lo(sbase + L::k(0, 0), 16);
-  const uint32_t v_lo = desc_lo(sbase + L::v(0, 0), kBox);
-  constexpr uint32_t kStage16 = (uint32_t)(L::kNB * kBox) >> 4;
-  // S_t = Q_t K^T: both operands K-major, 128-byte
-  // swizzle; a K step of 16 elements is 32 bytes inside a 64-column box.
-  auto qk = [&](int t, int st) {
-    const uint32_t a0 = q_lo + (uint32_t)(L::q(t, 0) >> 4);
-    const uint32_t b0 = k_lo + (uint32_t)st * kStage16;
-#pragma unroll
-    for (int ks = 0; ks < D / 16; ++ks) {
-      const uint32_t off = (uint32_t)((ks / 4) * kBox + (ks % 4) * 32) >> 4;
-      mma_ss_warp(tmem + T::s(t), a0 + off, b0 + off, hi, kIdescQK, ks > 0);
-    }
-  };
-  // O_t += P_t V: P_t from its TMEM columns (8 per 16 keys), V MN-major (d
-  // contiguous): 16 keys are two 8-row groups (2048 bytes), the two 64-column
-  // halves of d are one box apart.
-  auto pv = [&](int t, int st, int acc) {
-    const uint32_t b0 = v_lo + (uint32_t)st * kStage16;
-#pragma unroll
-    for (int kk = 0; kk < kBN / 16; ++kk)
-      mma_ts_warp(tmem + T::o(t), tmem + T::p(t) + kk * 8,
-                  b0 + (uint32_t)(kk * 2048 >> 4), hi, kIdescPV,
-                  (acc | kk) != 0);
-  };
-  // A QK^T may overwrite its S once the softmax warps have read the previous
-  // one into registers.  Shared S: the k-th QK^T (of either tile) waits for
-  // generation k - 1 of the one S barrier; own S: each tile has its barrier.
-  int s_uses[kQTiles] = {0, 0};
-  auto take_s = [&](int t) {
-    const int i = T::kOwnS ? t : 0;
-    if (s_uses[i]++ > 0) named_sync(i ? kBarSFree1 : kBarSFree);
-    tc_fence_after();
-  };
-
   // Test hook: o_full receives no arrival before the end of the stream, so
   // this wait runs out and exercises the abort path.
   bool ok = !p.inject_stall || wait_bar_warp(&S->o_full, 0, S, p.status);
   ok = ok && wait_bar_warp(&S->q_full, 0, S, p.status);
-  // Issue order per key tile j: QK_0(j), PV_0(j-1), QK_1(j), PV_1(j-1).  A
-  // tile's PV runs one key tile behind its QK^T, so the softmax of S_t(j)
-  // has the MMAs of three other steps (about 2000 clk) to produce P_t(j)
-  // before the pipe needs it, while S, which only has to survive until the
-  // softmax has loaded it, alternates between the tiles.
-  for (int j = 0; ok && j <= n; ++j) {
-    const bool has_qk = j < n;
-    const int st = j % kKStages;
-    const int jp = j - 1;  // the key tile whose PV runs now
-    const int vs = jp % kVStages;
-    if (has_qk) {
-      relay_sync(kBarKFull0 + st);
-      take_s(0);
-      qk(0, st);
-      mma_commit_warp(&S->s_full[0]);
-      if (!two) mma_commit_warp(&S->k_empty[st]);
-    }
-    if (jp >= 0) {
-      relay_sync(kBarVFull0 + vs);
-      named_sync(kBarPFull0);
-      tc_fence_after();
-      pv(0, vs, jp > 0);
-      mma_commit_warp(&S->p_free[0]);
-      if (!two) mma_commit_warp(&S->v_empty[vs]);
-    }
-    if (two) {
-      if (has_qk) {
-        take_s(1);
-        qk(1, st);
-        mma_commit_warp(&S->s_full[1]);
-        mma_commit_warp(&S->k_empty[st]);
-      }
-      if (jp >= 0) {
-        named_sync(kBarPFull0 + 1);
-        tc_fence_after();
-        pv(1, vs, jp > 0);
-        mma_commit_warp(&S->p_free[1]);
-        mma_commit_warp(&S->v_empty[vs]);
-      }
-    }
+  if (ok) {
+    MmaOps<D, true> ops{S, tmem, desc_hi_sw128(1024),
+                        desc_lo(sbase + L::q(0, 0), 16),
+                        desc_lo(sbase + L::k(0, 0), 16),
+                        desc_lo(sbase + L::v(0, 0), kBox)};
+    handoff::fwd_mma_steps(w.n, w.nqt == 2, Tmem<D>::kOwnS, ops);
+    mma_commit_warp(&S->o_full);
+  } else {
+    MmaOps<D, false> ops{S};
+    handoff::fwd_mma_steps(w.n, w.nqt == 2, Tmem<D>::kOwnS, ops);
   }
-  if (ok) mma_commit_warp(&S->o_full);
   mma_commit_warp(&S->drain);
   if ((threadIdx.x & 31) == 0) drain_wait(&S->drain, 0, S);
   __syncwarp();
@@ -650,17 +643,16 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
   const uint32_t tS = tmem + T::s(t) + lane_off;
   const uint32_t tP = tmem + T::p(t) + lane_off;
   const uint32_t tO = tmem + T::o(t) + lane_off;
-  const int bar_s = T::kOwnS && t ? kBarSFree1 : kBarSFree;
   const float sl2 = p.scale_log2;
   const uint64_t sl2x2 = f2_pack(sl2, sl2);
   float m_ref = -INFINITY;  // exp2-domain reference (scaled scores)
   float l = 0.f;
+  // Each wait is decided per warp, by a vote whose latency passes behind the
+  // loads or the exponentials that follow the wait: the TMEM accesses and the
+  // named barriers are warp-wide, so lanes must not part after a failed wait.
   bool ok = true;
-  // Arrivals the MMA warp waits for: one per S this tile reads, except the
-  // very last S of the unit (own S: of the tile; no QK^T follows it), and one
-  // per P_t.
-  const int s_expected = (T::kOwnS || t == nqt - 1) ? n - 1 : n;
-  int s_arrived = 0, p_arrived = 0;
+  const int s_expected = handoff::fwd_s_arrivals(n, t, nqt, T::kOwnS);
+  int s_done = n;  // "S read" arrivals made
   int vis_lo = 0, vis_hi = 0;  // one-shot: this row's visible key tokens
   if (kOneShot) {
     const int row = min(q0 + t * kBM + wq * 32 + lane, p.q_tokens - 1);
@@ -677,7 +669,8 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
   const int rag0_n = p.seg_len[0] % kBN, rag1_n = p.seg_len[1] % kBN;
   const int rag0 = rag0_n ? p.seg_tiles0 - 1 - j0 : -1;
   const int rag1 = rag1_n ? p.total_tiles - 1 - j0 : -1;
-  for (int j = 0; j < n; ++j) {
+  int j = 0;  // and, after the loop, "P stored" arrivals made
+  for (; j < n; ++j) {
     const int jt = rev ? n - 1 - j : j;  // the producers' order
     int lo = 0, hi = kBN;  // the columns of the tile that the row sees
     bool masked;
@@ -691,18 +684,20 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
       if (jt == rag0) hi = rag0_n;
       if (jt == rag1) hi = rag1_n;
     }
-    if (!(ok = wait_bar(&S->s_full[t], j & 1, S, p.status))) break;
+    const bool s_ok = wait_bar(&S->s_full[t], j & 1, S, p.status);
     tc_fence_after();
     uint32_t s[4][32];
 #pragma unroll
     for (int c = 0; c < 4; ++c) tmem_ld32(tS + 32 * c, s[c]);
+    ok = __all_sync(0xffffffffu, s_ok);
     tmem_wait_ld();
+    if (!ok) {
+      s_done = j;
+      break;
+    }
     // S is in registers: the next QK^T (of either tile) may overwrite it.
     tc_fence_before();
-    if (s_arrived < s_expected) {
-      named_arrive(bar_s);
-      ++s_arrived;
-    }
+    if (j < s_expected) named_arrive(handoff::fwd_s_free(t, T::kOwnS));
     // At d = 64 the softmax warps set the pace (about 2000 clk per key tile
     // against 1170 of MMAs): a first look at p_free is sent off here, so that
     // its latency passes behind the row max.  At d = 128 it gained nothing.
@@ -737,9 +732,8 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
     for (int c = 0; c < 2; ++c) exp_pack32(s[c], sl2x2, neg2, pk[c], acc);
     // P_t(j - 1) has been consumed and O_t holds PV_t(0 .. j-1) (PV_t(j-1)
     // was issued right after this S, so this normally does not wait).
-    if (j > 0 && !p_is_free &&
-        !(ok = wait_bar(&S->p_free[t], (j - 1) & 1, S, p.status)))
-      break;
+    const bool p_ok = j == 0 || p_is_free ||
+                      wait_bar(&S->p_free[t], (j - 1) & 1, S, p.status);
     tc_fence_after();
     if (rescale && j > 0) {
       // Scale O_t in place before PV_t(j) accumulates against the new
@@ -763,23 +757,32 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
       tmem_st16(tP + 16 * c, pk[c - 2]);
     }
     l += acc_total(acc);
+    ok = __all_sync(0xffffffffu, p_ok);
     tmem_wait_st();
     tc_fence_before();
-    named_arrive(kBarPFull0 + t);
-    ++p_arrived;
+    if (!ok) {
+      s_done = j + 1;
+      break;
+    }
+    named_arrive(handoff::fwd_p_full(t));
   }
-  // After a failed wait the remaining hand-offs are still made (their
-  // contents are undefined, and so is the output), so that the MMA warp
-  // never waits for an arrival that does not come.
-  while (s_arrived < s_expected) {
-    named_arrive(bar_s);
-    ++s_arrived;
+  if (!ok) {
+    struct Ops {
+      Shared* S;
+      int t;
+      OwedWaits owed;
+      __device__ __forceinline__ void wait_s(int j) {
+        owed.wait(&S->s_full[t], j & 1);
+      }
+      __device__ __forceinline__ void wait_p(int j) {
+        owed.wait(&S->p_free[t], j & 1);
+      }
+      __device__ __forceinline__ void arrive(int id) { named_arrive(id); }
+    };
+    handoff::fwd_softmax_rest(n, t, T::kOwnS, s_expected, s_done, j,
+                              Ops{S, t, {}});
   }
-  while (p_arrived < n) {
-    named_arrive(kBarPFull0 + t);
-    ++p_arrived;
-  }
-  const bool have = ok && wait_bar(&S->o_full, 0, S, p.status);
+  const bool have = ok && wait_bar_warp(&S->o_full, 0, S, p.status);
   const Work w = cta_work<kOneShot>(p);
   const int r_unit = t * kBM + wq * 32 + lane;  // row within the unit
   const int row = w.q0 + r_unit;
