@@ -50,6 +50,7 @@
 // loads and MMAs are drained, TMEM is released and the CTA exits.
 #include <cuda.h>
 #include <cuda_bf16.h>
+#include <float.h>
 #include <math.h>
 
 #include <algorithm>
@@ -629,7 +630,7 @@ __device__ __forceinline__ void max32(const uint32_t (&sc)[32],
 
 // Streaming: j0, n index the launch's visible tiles.  One-shot: the tiles of
 // [kv0, kv1); a row of chunk c sees keys of chunks max(0, c - W) .. c, so a
-// row can be fully masked in a tile (its reference then stays at -inf).
+// row can be fully masked in a tile (its reference then stays as it was).
 // Per key tile: read S (shared by both query tiles) into registers and
 // release it at once, exponentiate, wait until the previous PV of this tile
 // has consumed P_t (and brought O_t up to date), rescale O_t if the
@@ -645,7 +646,11 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
   const uint32_t tO = tmem + T::o(t) + lane_off;
   const float sl2 = p.scale_log2;
   const uint64_t sl2x2 = f2_pack(sl2, sl2);
-  float m_ref = -INFINITY;  // exp2-domain reference (scaled scores)
+  // exp2-domain reference (scaled scores).  It starts at the lowest finite
+  // value: a row that has seen no visible key yet, or none with a score above
+  // -inf (one that overflowed), then exponentiates -inf, to 0, and not
+  // -inf + inf.
+  float m_ref = -FLT_MAX;
   float l = 0.f;
   // Each wait is decided per warp, by a vote whose latency passes behind the
   // loads or the exponentials that follow the wait: the TMEM accesses and the
@@ -719,13 +724,10 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
     if (rescale) {
       const float m_new = fmaxf(m_ref, mrow);
       alpha = ex2(m_ref - m_new);
-      if (kOneShot && m_new == -INFINITY) alpha = 1.f;  // still nothing seen
       l *= alpha;
       m_ref = m_new;
     }
-    // A row that has seen no visible key yet exponentiates -inf against 0.
-    const float neg = (kOneShot && m_ref == -INFINITY) ? 0.f : -m_ref;
-    const uint64_t neg2 = f2_pack(neg, neg);
+    const uint64_t neg2 = f2_pack(-m_ref, -m_ref);
     uint64_t acc[4] = {0, 0, 0, 0};
     uint32_t pk[2][16];
 #pragma unroll
@@ -786,7 +788,9 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
   const Work w = cta_work<kOneShot>(p);
   const int r_unit = t * kBM + wq * 32 + lane;  // row within the unit
   const int row = w.q0 + r_unit;
-  const float inv_l = 1.f / l;
+  // A part may hold nothing but scores of -inf for a row: its O is then 0, and
+  // its log-sum-exp of -inf gives it no weight in the merge.  (A NaN l stays.)
+  const float inv_l = w.part >= 0 && l == 0.f ? 0.f : 1.f / l;
   if (w.part >= 0) {
     // Partial result of a key range: O / l in fp32 (transposed, so a warp's
     // stores are contiguous) and the log2-domain log-sum-exp.
@@ -997,7 +1001,8 @@ combine_few_kernel(const __grid_constant__ TcParams p) {
   for (int u = 0; u < kFewParts; ++u)
 #pragma unroll
     for (int r = 0; r < 4; ++r) {
-      w[u][r] = ex2(w[u][r] - m[r]);  // 0 for the missing parts
+      // 0 for the missing parts, and where no part has anything finite
+      w[u][r] = ex2(w[u][r] - (m[r] == -INFINITY ? 0.f : m[r]));
       wsum[r] += w[u][r];
     }
   float acc[kFewCols][4] = {};

@@ -145,6 +145,51 @@ def test_work_split_shapes(w):
     run_stream(w, rows_per_chunk=48).check()
 
 
+# Scores that overflow to -inf in fp32 (q . k below -2^128; float64 holds them)
+# carry no weight, wherever they lie: in the first key tile that a unit or a part
+# of one walks, in a whole part, in the last tiles.  Every second query row has
+# them on the poisoned keys; the other rows see ordinary scores.
+POISONED = {
+    "first": lambda t, n: t < n - 64,        # all but the last 64 keys
+    "last": lambda t, n: t >= 64,            # all but the first 64 keys
+    "even-tiles": lambda t, n: t // 128 % 2 == 0,
+    "odd-tiles": lambda t, n: (t // 128 % 2 == 1) | (t >= n // 128 * 128),
+}
+OVERFLOW = [
+    # whole units of one query tile, of two; equal parts of few units
+    # (combine_kernel); two unequal parts (combine_few_kernel), both head dims
+    SMALL[0],
+    WL.custom("two-tiles", batch=1, heads=80, head_dim=64,
+              tokens_per_frame=260, frames_per_chunk=1, num_chunks=2, seed=91),
+    SMALL[7], SPLITS[0],
+    WL.custom("unequal-parts-d128", batch=1, heads=17, head_dim=128,
+              tokens_per_frame=1120, frames_per_chunk=1, num_chunks=3, seed=92),
+]
+
+
+@pytest.mark.parametrize("pattern", POISONED)
+@pytest.mark.parametrize("w", OVERFLOW, ids=lambda w: w.name)
+def test_scores_of_minus_infinity_carry_no_weight(FV, w, pattern):
+    att = FV.StreamingAttention(FV.config_from_workload(w))
+    ks, vs, at = [], [], 0
+    for c, q, k, v in WL.chunk_stream(w):
+        t = torch.arange(at, at + k.shape[1])
+        at += k.shape[1]
+        poison = POISONED[pattern](t, w.num_tokens)
+        k[..., 0] = torch.where(poison, -2.0 ** 65, 0.0)[None, :, None]
+        q[..., 0] = 0
+        q[:, ::2, :, 0] = 2.0 ** 65
+        att.append(k.cuda(), v.cuda())
+        ks.append(k), vs.append(v)
+    o, lse = att.forward(q.cuda(), want_lse=True)
+    rows = np.unique(np.linspace(0, q.shape[1] - 1, 40).astype(int))
+    ref_o, ref_l = OA.chunk_attention(to64(q[:, rows]), to64(torch.cat(ks, 1)),
+                                      to64(torch.cat(vs, 1)), w.softmax_scale)
+    err = Err()
+    err.add(to64(o.cpu()[:, rows]), ref_o, lse.cpu().numpy()[:, :, rows], ref_l)
+    err.check()
+
+
 @pytest.mark.parametrize("w", SMALL[:3], ids=lambda w: w.name)
 def test_streamed_gpu_equals_oneshot_oracle(FV, w):
     att = FV.StreamingAttention(FV.config_from_workload(w))
