@@ -16,10 +16,19 @@ import ctypes
 import os
 from typing import Optional, Tuple
 
-try:  # only the torch conveniences below need it
-    import torch
-except ImportError:
-    torch = None
+
+class _TorchAtFirstUse:
+    """Stands in for torch until one of the conveniences below uses it: the
+    C-named calls need no torch, nor the seconds that its import takes.  The
+    module then takes this object's place, so later uses cost nothing."""
+
+    def __getattr__(self, name):
+        import torch as module
+        globals()["torch"] = module
+        return getattr(module, name)
+
+
+torch = _TorchAtFirstUse()
 
 _HERE = os.path.dirname(os.path.abspath(__file__))
 LIB_PATH = os.path.join(_HERE, "libfastvr_attn.so")
@@ -125,17 +134,19 @@ def _current_stream() -> int:
     """cudaStream_t of torch's current stream on the current device.  A small
     call is bound by its host time, and building a torch.cuda.Stream object
     for its handle took 2.8 us of it; the raw handle takes 0.1."""
+    global _raw_stream, _current_device
+    if _raw_stream is None:
+        c = torch._C
+        if hasattr(c, "_cuda_getCurrentRawStream") and hasattr(c, "_cuda_getDevice"):
+            _current_device = c._cuda_getDevice
+            _raw_stream = c._cuda_getCurrentRawStream
+        else:
+            _current_device = lambda: None
+            _raw_stream = lambda _: torch.cuda.current_stream().cuda_stream
     return _raw_stream(_current_device())
 
 
-def _stream_handle(_device: int) -> int:
-    return torch.cuda.current_stream().cuda_stream
-
-
-_raw_stream = getattr(getattr(torch, "_C", None), "_cuda_getCurrentRawStream",
-                      _stream_handle)
-_current_device = getattr(getattr(torch, "_C", None), "_cuda_getDevice",
-                          lambda: 0)
+_raw_stream = _current_device = None  # torch's calls, looked up at first use
 
 
 # ------------------------------------------------------------ C-named calls

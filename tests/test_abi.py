@@ -4,6 +4,8 @@ matches the oracle's definition of visibility.  No compute call runs here."""
 import ctypes
 import os
 import re
+import subprocess
+import sys
 
 import numpy as np
 import pytest
@@ -275,3 +277,32 @@ def test_static_entry_rejects_bad_arguments_before_any_device_work(fv):
         fv.fastvr_chunk_attn_fwd_static(bad_d, FAKE, 1, FAKE, FAKE, 256, ok_seg,
                                         FAKE, 0, 0)
     assert e.value.status == fv.FASTVR_ERR_UNSUPPORTED
+
+
+BINDING_WITHOUT_TORCH = """
+import sys
+sys.path[:0] = {paths!r}
+from paper_2609_36757_gb300 import fastvr as FV
+assert not any(m == "torch" or m.startswith("torch.") for m in sys.modules)
+cfg = FV.make_config(1, 2, 64, 4, 2, 1, 0)
+need = FV.fastvr_kv_cache_bytes(cfg)
+plan = FV.fastvr_attn_plan(cfg, 1 << 40, need)
+FV.fastvr_plan_destroy(plan)
+try:
+    FV.StreamingAttention(cfg)
+except {error} as e:
+    assert "broken here" in str(e)
+else:
+    raise AssertionError("the convenience class needs torch")
+"""
+
+
+@pytest.mark.parametrize("error", ["ImportError", "OSError", "RuntimeError"])
+def test_c_named_calls_need_no_torch(fv, tmp_path, error):
+    # a torch that cannot be imported (a missing shared library is an OSError)
+    # costs the C-named calls nothing, and is reported by the calls that use it
+    (tmp_path / "torch.py").write_text(f"raise {error}('torch is broken here')\n")
+    code = BINDING_WITHOUT_TORCH.format(paths=[str(tmp_path), ROOT], error=error)
+    r = subprocess.run([sys.executable, "-c", code], capture_output=True,
+                       text=True)
+    assert r.returncode == 0, r.stderr
