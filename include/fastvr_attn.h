@@ -243,7 +243,8 @@ FASTVR_API fastvr_status_t fastvr_one_step_update(const void* z_lq,
  *            head's cache, as fastvr_plan_visible reports them
  *   out      bf16 [B, q_frames*N, H, d]; lse nullable, float32 [B, H, Lq]
  * The result equals fastvr_chunk_attn_fwd's for the same inputs (same
- * kernels, same work split).  The first call on each device resolves the
+ * kernels, same work split: both leave at most as many partial results as the
+ * array holds, 190 at d = 128, or 256).  The first call on each device resolves the
  * array's device address (a symbol lookup, no allocation): make that first
  * call before any stream capture.  Every call on a device shares the array
  * and it keeps the last call's contents (nothing in it needs clearing:
@@ -254,9 +255,7 @@ FASTVR_API fastvr_status_t fastvr_one_step_update(const void* z_lq,
  * called.  Limits: q_frames * N and every seg_start + seg_len at most
  * 2^30 - 1 (the kernels index tokens in 32 bits); softmax_scale finite.
  * Errors: INVALID_ARG (null or misaligned pointers, bad sizes or ranges),
- * UNSUPPORTED (head_dim, device not sm_103), CAPACITY (the call's split
- * needs more partial results than the array holds: 190 at d = 128, 378 at
- * d = 64), CUDA. */
+ * UNSUPPORTED (head_dim, device not sm_103), CUDA. */
 FASTVR_API fastvr_status_t fastvr_chunk_attn_fwd_static(
     const fastvr_attn_config_t* cfg, const void* q, int32_t q_frames,
     const void* k_cache, const void* v_cache, int64_t cache_tokens,

@@ -1196,12 +1196,6 @@ int long_pairs(int q_tokens) {
   return (q_tokens + kBM - 1) / (kQTiles * kBM);
 }
 
-int total_tiles(const AttnParams& a) {
-  int tiles = 0;
-  for (int s = 0; s < a.num_segments; ++s) tiles += (a.seg_len[s] + kBN - 1) / kBN;
-  return tiles;
-}
-
 bool make_map(CUtensorMap* m, const void* base, int d, int64_t tokens,
               int heads, int batch, int64_t token_stride_b,
               int64_t head_stride_b, int64_t batch_stride_b) {
@@ -1367,15 +1361,6 @@ cudaError_t launch_blockcausal_attn(const OneShotParams& p, cudaStream_t stream)
   if (p.head_dim == 64) return launch_oneshot_d<64>(p, stream);
   if (p.head_dim == 128) return launch_oneshot_d<128>(p, stream);
   return cudaErrorInvalidValue;
-}
-
-int chunk_attn_parts(const AttnParams& a) {
-  const int bh = a.heads * a.batch;
-  const int units = units_of(a.q_tokens, kUnitRows) * bh;
-  const Split sp = split_units(units, units_of(a.q_tokens, kBM) * bh,
-                               total_tiles(a), sm_count(),
-                               split_parts(a.head_dim));
-  return sp.split > 1 ? (units - sp.units_full) * sp.split : 0;
 }
 
 cudaError_t launch_chunk_attn(const AttnParams& p, cudaStream_t stream,

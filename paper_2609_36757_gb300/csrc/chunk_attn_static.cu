@@ -28,8 +28,8 @@
 
 namespace {
 
-// 24 MiB: room for 190 partial results at d = 128 (378 at d = 64); a launch
-// leaves at most 190 (256 at d = 64), see split_parts.
+// 24 MiB, which bounds every launch's partial results (split_parts): 190 at
+// d = 128, 256 at d = 64.
 constexpr size_t kScratchBytes = fastvr::kStaticScratchBytes;
 
 static __device__ __align__(256) unsigned char g_scratch[kScratchBytes];
@@ -146,14 +146,10 @@ extern "C" fastvr_status_t fastvr_chunk_attn_fwd_static(
       cfg->softmax_scale == 0.f ? 1.f / sqrtf((float)d) : cfg->softmax_scale;
   a.scale_log2 = scale * 1.4426950408889634f;
 
-  // The array holds partial results only.  A call whose split needs more of
-  // them than fit is refused rather than run with a different split.  The
-  // array keeps the last call's contents, which needs no clearing: every
-  // partial result is written before it is read.
-  const int capacity = (int)(kScratchBytes / fastvr::part_bytes(d));
-  if (fastvr::chunk_attn_parts(a) > capacity) return FASTVR_ERR_CAPACITY;
+  // The array holds partial results only, and it keeps the last call's, which
+  // need no clearing: every partial result is written before it is read.
   a.workspace = reinterpret_cast<float*>(scratch);
-  a.workspace_parts = capacity;
+  a.workspace_parts = fastvr::split_parts(d);
   // Timeouts go to the sticky per-device word (zero at load, cleared when
   // fastvr_get_device_status reads it).
   a.status = fastvr::device_status_word();

@@ -15,13 +15,14 @@ namespace fastvr {
 // Sec. 3.1 KV caching).
 constexpr int kMaxSegments = 2;
 
-// Split-KV workspace of the attention kernel: at most kMaxParts partial
-// results of 256 query rows, each d fp32 outputs plus one log-sum-exp.
+// Split-KV workspace of a plan: kMaxParts partial results of 256 query rows,
+// each d fp32 outputs plus one log-sum-exp.
 constexpr int kMaxParts = 256;
 constexpr int kUnitRows = 256;
 // Scratch array of the allocation-free entry point, and the most partial
 // results that any launch leaves: what fits both it and the plan's workspace,
-// so that the two entry points split the same work the same way.
+// so that the two entry points split the same work the same way (190 at
+// d = 128, 256 at d = 64).
 constexpr size_t kStaticScratchBytes = size_t(24) << 20;
 constexpr size_t part_bytes(int head_dim) {
   return (size_t)kUnitRows * (head_dim + 1) * sizeof(float);
@@ -31,6 +32,10 @@ constexpr int split_parts(int head_dim) {
              ? (int)(kStaticScratchBytes / part_bytes(head_dim))
              : kMaxParts;
 }
+static_assert(split_parts(64) <= kMaxParts && split_parts(128) <= kMaxParts &&
+                  split_parts(64) * part_bytes(64) <= kStaticScratchBytes &&
+                  split_parts(128) * part_bytes(128) <= kStaticScratchBytes,
+              "a launch's partial results fit both workspaces");
 inline size_t workspace_bytes(int head_dim) {
   return (size_t)kMaxParts * kUnitRows * (head_dim + 1) * sizeof(float);
 }
@@ -140,7 +145,8 @@ struct AttnParams {
   float scale_log2;       // softmax_scale * log2(e)
   int* status;            // control word (device)
   float* workspace;       // split-KV scratch (device): workspace_parts
-                          // partial results of kUnitRows x (d + 1) floats
+                          // partial results of kUnitRows x (d + 1) floats,
+                          // at least split_parts(d) of them
   int32_t workspace_parts;
   uint64_t wait_limit_ns; // bound of every in-kernel wait (0 = default)
   int32_t inject_stall;   // test hook: stall the MMA issuer until timeout
@@ -188,9 +194,6 @@ cudaError_t launch_blockcausal_attn_bwd(const BwdArgs& a, cudaStream_t stream);
 // one-shot forward and the backward), or null if it cannot be looked up.
 int* device_status_word();
 
-// Workspace parts (partial results) a launch of p uses on the current device
-// (0 when no unit is split), with at most kMaxParts parts.
-int chunk_attn_parts(const AttnParams& p);
 // Enqueues the attention kernel (and the merge kernel when the key range of
 // some units is split); *launches receives the number of kernels enqueued.
 cudaError_t launch_chunk_attn(const AttnParams& p, cudaStream_t stream,
