@@ -39,14 +39,15 @@ class Err:
             lse_got: Optional[np.ndarray] = None,
             lse_ref: Optional[np.ndarray] = None) -> None:
         d = np.abs(got.astype(np.float64) - ref)
-        self.max_abs = max(self.max_abs, float(d.max()) if d.size else 0.0)
+        # np.maximum keeps a NaN, max() would drop it
+        self.max_abs = float(np.maximum(self.max_abs, d.max() if d.size else 0.0))
         self.sum_abs += float(d.sum())
         self.count += d.size
         self.sq_err += float((d * d).sum())
         self.sq_ref += float((ref * ref).sum())
         if lse_got is not None:
-            self.lse_max = max(self.lse_max, float(
-                np.abs(lse_got.astype(np.float64) - lse_ref).max()))
+            self.lse_max = float(np.maximum(
+                self.lse_max, np.abs(lse_got.astype(np.float64) - lse_ref).max()))
 
     @property
     def mean_abs(self) -> float:

@@ -3,11 +3,12 @@ oracle's own on the same bf16 values (the 16-bit patterns are widened to
 float64 exactly), so the pool changes where the oracle runs, not what it
 computes."""
 import numpy as np
+import pytest
 import torch
 
 import oracle_pool
 from oracle import attention as OA
-from parity_helpers import bf16_bits, to64
+from parity_helpers import Err, bf16_bits, to64
 
 
 def test_bf16_widening_is_exact():
@@ -33,3 +34,15 @@ def test_pool_rows_equal_the_serial_oracle():
         o, lse = OA.softmax_attention(to64(q), to64(k), to64(v), 0.125)
         np.testing.assert_allclose(results[i][0], o, rtol=0, atol=1e-12)
         np.testing.assert_allclose(results[i][1], lse, rtol=0, atol=1e-12)
+
+
+@pytest.mark.parametrize("where", ["output", "lse"])
+def test_the_parity_check_sees_a_nan(where):
+    ref_o, ref_l = np.ones((2, 4)), np.ones((2,))
+    o, lse = ref_o.copy(), ref_l.copy()
+    (o if where == "output" else lse).flat[1] = np.nan
+    err = Err()
+    err.add(o, ref_o, lse, ref_l)
+    err.add(ref_o, ref_o, ref_l, ref_l)
+    with pytest.raises(AssertionError):
+        err.check()
