@@ -23,6 +23,22 @@ CASES = [
     WL.custom("d64-N130-W2", batch=1, heads=4, head_dim=64,
               tokens_per_frame=130, frames_per_chunk=2, num_chunks=5,
               window_chunks=2, last_chunk_frames=1, seed=23),
+    # the three above run units of one query tile, or parts that combine_kernel
+    # merges; whole units of two query tiles, the short ones behind the others
+    WL.custom("two-tiles-d128", batch=1, heads=80, head_dim=128,
+              tokens_per_frame=260, frames_per_chunk=1, num_chunks=3, seed=32),
+    # the same over a wrapped ring, both segments ragged
+    WL.custom("two-tiles-ring-d64", batch=2, heads=40, head_dim=64,
+              tokens_per_frame=130, frames_per_chunk=2, num_chunks=7,
+              window_chunks=2, last_chunk_frames=1, seed=33),
+    # combine_few_kernel: two unequal parts, and three equal ones behind a wave
+    WL.custom("unequal-parts-d64", batch=1, heads=17, head_dim=64,
+              tokens_per_frame=1120, frames_per_chunk=1, num_chunks=5, seed=34),
+    WL.custom("few-parts-d128", batch=1, heads=64, head_dim=128,
+              tokens_per_frame=600, frames_per_chunk=1, num_chunks=3, seed=35),
+    # a wave of long and short units, then short ones in parts
+    WL.custom("short-tail-d128", batch=1, heads=33, head_dim=128,
+              tokens_per_frame=1100, frames_per_chunk=1, num_chunks=3, seed=36),
 ]
 
 

@@ -137,6 +137,20 @@ SPLITS = [
     WL.custom("short-in-place", batch=1, heads=3, head_dim=64,
               tokens_per_frame=16500, frames_per_chunk=1, num_chunks=2,
               seed=85),
+    # 40 units behind a whole wave, three equal parts each: the merge of few
+    WL.custom("few-parts", batch=1, heads=64, head_dim=128,
+              tokens_per_frame=600, frames_per_chunk=1, num_chunks=3, seed=86),
+    # 95 units of up to 50 tiles, two unequal parts each: 190 partial results,
+    # all that the scratch holds at d = 128; and 96, which run whole for it
+    WL.custom("95-units-d128", batch=1, heads=19, head_dim=128,
+              tokens_per_frame=1280, frames_per_chunk=1, num_chunks=5, seed=87),
+    WL.custom("96-units-d128", batch=1, heads=24, head_dim=128,
+              tokens_per_frame=1024, frames_per_chunk=1, num_chunks=6, seed=88),
+    # whole units of two query tiles over a ring that has wrapped, both
+    # segments ragged
+    WL.custom("ring-two-tiles", batch=2, heads=40, head_dim=64,
+              tokens_per_frame=130, frames_per_chunk=2, num_chunks=7,
+              window_chunks=2, last_chunk_frames=1, seed=89),
 ]
 
 
@@ -158,12 +172,13 @@ POISONED = {
 OVERFLOW = [
     # whole units of one query tile, of two; equal parts of few units
     # (combine_kernel); two unequal parts (combine_few_kernel), both head dims
-    SMALL[0],
+    WL.custom("one-tile", batch=1, heads=8, head_dim=128, tokens_per_frame=130,
+              frames_per_chunk=1, num_chunks=5, seed=90),
     WL.custom("two-tiles", batch=1, heads=80, head_dim=64,
               tokens_per_frame=260, frames_per_chunk=1, num_chunks=2, seed=91),
     SMALL[7], SPLITS[0],
     WL.custom("unequal-parts-d128", batch=1, heads=17, head_dim=128,
-              tokens_per_frame=1120, frames_per_chunk=1, num_chunks=3, seed=92),
+              tokens_per_frame=1120, frames_per_chunk=1, num_chunks=5, seed=92),
 ]
 
 
@@ -247,6 +262,17 @@ def test_forward_is_deterministic_and_repeatable(FV):
         o1 = att.forward(qd)
         o2 = att.forward(qd)
         assert torch.equal(o1, o2)
+
+
+@pytest.mark.parametrize("w", SPLITS, ids=lambda w: w.name)
+def test_split_launches_are_deterministic(FV, w):
+    att = FV.StreamingAttention(FV.config_from_workload(w))
+    for c, q, k, v in WL.chunk_stream(w):
+        att.append(k.cuda(), v.cuda())
+    qd = q.cuda()
+    o1, l1 = att.forward(qd, want_lse=True)
+    o2, l2 = att.forward(qd, want_lse=True)
+    assert torch.equal(o1, o2) and torch.equal(l1, l2)
 
 
 def test_errors_on_the_gpu_path(FV):
