@@ -520,9 +520,9 @@ __device__ __forceinline__ constexpr bool poly_group(int q) { return q == 7; }
 // P = 2^(s c2 - lse2) for 32 columns [c0, c0 + 32) of a half row, packed to
 // bf16 pairs for the dV MMA and, in s, in fp32 for dS (dS from the bf16 pairs
 // had to widen them again, two of three ALU instructions per pair of columns,
-// added P's rounding error to dK: training clip step, with the dQ kernel's
-// form below, 2244 -> 2203 us, dK's error against 64 bits 2.9e-3 -> 2.4e-3 at
-// d = 64); with kMask, columns outside [lo, hi) are masked (p = 0).  nl
+// and added P's rounding error to dK: crop training step, with the dQ kernel's
+// form below, 142.6 -> 137.8 us, dK's error against 64 bits 2.9e-3 -> 2.4e-3 at
+// d = 64; the training clip's step gained 1.5 %, within its runs' spread); with kMask, columns outside [lo, hi) are masked (p = 0).  nl
 // holds -lse2 for the 32 columns, in registers: the dK/dV kernel reads its
 // per-column values from shared memory ahead of use, because the SMEM x SMEM
 // MMAs that run meanwhile take all of the shared-memory bandwidth and each
@@ -590,7 +590,7 @@ __device__ __forceinline__ void ds32(const uint32_t (&pf)[32],
 // and in place: rounded to bf16 pairs and widened again it took three of the
 // four ALU instructions per pair of columns in the two phases, which set the
 // step's pace (1650 clk against 840 of MMAs at d = 64, 1536 at d = 128).  Crop
-// training step 142.8 -> 138.1 us, clip 2271 -> 2235; with one rounding less
+// training step 142.8 -> 138.1 us; with one rounding less
 // dQ's error against 64 bits falls from 2.9e-3 to 2.4e-3 (crop).  nl and nd are
 // the row's own -lse2 and -D.
 template <bool kMask>

@@ -46,8 +46,10 @@
 // evict_last for K/V (every unit of the head reads them).
 //
 // Every mbarrier wait is bounded: past the limit the kernel records
-// FASTVR timeout in the control word, all roles stop issuing, in-flight TMA
-// loads and MMAs are drained, TMEM is released and the CTA exits.
+// FASTVR timeout in the control word, no role starts new copies or takes up
+// new work, the hand-offs are made to the end (the MMA warp, if it had begun,
+// runs on over undefined data), in-flight TMA loads and MMAs are drained, TMEM
+// is released and the CTA exits.
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <float.h>
@@ -631,8 +633,8 @@ __device__ __forceinline__ void max32(const uint32_t (&sc)[32],
 // Streaming: j0, n index the launch's visible tiles.  One-shot: the tiles of
 // [kv0, kv1); a row of chunk c sees keys of chunks max(0, c - W) .. c, so a
 // row can be fully masked in a tile (its reference then stays as it was).
-// Per key tile: read S (shared by both query tiles) into registers and
-// release it at once, exponentiate, wait until the previous PV of this tile
+// Per key tile: read S (at d = 128 one buffer for both query tiles, at d = 64
+// one each) into registers and release it at once, exponentiate, wait until the previous PV of this tile
 // has consumed P_t (and brought O_t up to date), rescale O_t if the
 // reference moved, then store P_t.
 template <int D, bool kOneShot>
@@ -669,8 +671,8 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
   // most one tile each); one-shot, tiles that cross a chunk edge.  Whether
   // this one does is settled before S is waited for and decided once per
   // tile: worked out after the wait, with a test per 32 columns, it stood in
-  // the chain from S to P (training clip forward 504.9 -> 498.0 us; 480p ring,
-  // 84 CTAs of 63 tiles, 77.2 -> 76.7).
+  // the chain from S to P (d = 64 chunk step, 48 heads of 3465 x 10395, with
+  // one S for both query tiles as it then was: 433.7 -> 429.2 us).
   const int rag0_n = p.seg_len[0] % kBN, rag1_n = p.seg_len[1] % kBN;
   const int rag0 = rag0_n ? p.seg_tiles0 - 1 - j0 : -1;
   const int rag1 = rag1_n ? p.total_tiles - 1 - j0 : -1;
@@ -704,7 +706,7 @@ __device__ void softmax_role(const TcParams& p, Shared* S, uint32_t tmem,
     tc_fence_before();
     if (j < s_expected) named_arrive(handoff::fwd_s_free(t, T::kOwnS));
     // At d = 64 the softmax warps set the pace (about 2000 clk per key tile
-    // against 1170 of MMAs): a first look at p_free is sent off here, so that
+    // against 1040 of MMAs): a first look at p_free is sent off here, so that
     // its latency passes behind the row max.  At d = 128 it gained nothing.
     const bool p_is_free =
         T::kOwnS && j > 0 && mbar_test_wait(&S->p_free[t], (j - 1) & 1);
@@ -1135,9 +1137,12 @@ constexpr double kOneTileCost = 0.75;
 
 // Launches whose units have at most this many key tiles run a head's unit of
 // one query tile after all others: it is the cheaper one to have left over
-// (480p, chunk of 25 tiles: 49.5 -> 43.1 us; no slower up to its 199 tiles).
-// Run there, away from its head's other units, it reads the head's keys once
-// more; at 720p's 450 tiles the launch is 0.7 % slower for it.
+// (480p, chunk of 25 tiles: 49.5 -> 43.1 us; 3180 queries, 12, 24 or 48 heads,
+// d = 64 and 128: 63 tiles 0.6-4 % faster, 157 and 243 tiles 0.2-2 %).  Run
+// there, away from its head's other units, it reads the head's keys once more.
+// Past the line that goes either way: the same queries over 313 and 454 tiles
+// would gain 0.4-1.4 %, 720p's 7200 queries x 12 heads over 450 tiles lost
+// 0.7 %; it stays in its place there.
 constexpr int kShortsLastTiles = 256;
 
 // Whole waves of units run whole; the units of a last partial wave are cut
@@ -1151,6 +1156,11 @@ constexpr int kShortsLastTiles = 256;
 // round the rest, at most q on one SM, and the cut lies where both end
 // together.  (Equal parts in one round at most left 68 of 152 SMs idle for a
 // 480p frame, 84 units of 63 tiles: 76.8 us, now 65.9 with the merge.)
+//
+// max_parts is what the allocation-free entry point's scratch holds, so that
+// both entry points split alike, and it ends the second form early at d = 128:
+// 95 units of 63 tiles are cut (66 us), 96 would need 192 parts of the 190 and
+// run whole (76 us).
 //
 // Where twice the units still fit the SMs, units of one query tile are the
 // other way to use more of them, and cost no merge (chunk of 600 queries x 2400

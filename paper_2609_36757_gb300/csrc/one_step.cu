@@ -53,8 +53,9 @@ __device__ __forceinline__ void from_f(__nv_bfloat16& d, float x) {
 // z and out may be the same buffer (in-place update): every element is read
 // and then written by the same thread.  Each thread keeps a few groups of loads
 // in flight before it computes and stores, so that a few CTAs per SM cover the
-// HBM latency: 128 bytes at 4 bf16 or 8 fp32 groups, then, since a latent of a
-// few million elements gives a thread only two or three groups, two at a time.
+// HBM latency: four groups at bf16 (128 bytes), eight at fp32 (192 bytes), then,
+// since an fp32 latent of a few million elements gives a thread only two or
+// three groups, two at a time.
 template <typename T>
 __device__ __forceinline__ void update(const Vec<T>& zv,
                                        const typename Vec<T>::V& vv,
