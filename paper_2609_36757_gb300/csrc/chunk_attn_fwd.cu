@@ -417,10 +417,12 @@ struct OwedWaits {
 // A commit of the MMA warp; with nothing issued, an arrival.
 template <bool kIssue>
 __device__ __forceinline__ void commit_step(uint64_t* bar) {
-  if (kIssue)
+  if (kIssue) {
     mma_commit_warp(bar);
-  else if ((threadIdx.x & 31) == 0)
-    mbar_arrive(bar);
+  } else {
+    if ((threadIdx.x & 31) == 0) mbar_arrive(bar);
+    __syncwarp();  // converged at the next named barrier
+  }
 }
 
 // Hand-offs from the softmax warps to the MMA warp go through named
